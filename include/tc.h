@@ -65,14 +65,19 @@ enum {                      /* field selector of tc_get_field / tc_set_field */
 enum { TC_SPECTRAL = 0, TC_PHYSICAL = 1 };
 
 enum {
-    TC_PREC_FP64 = 0,       /* every step in float64 */
+    TC_PREC_FP64 = 0,       /* every step in float64, the transforms and products
+                               in 64-bit fixed point with one scale per
+                               transform (error below float64's) where the
+                               padded lengths are at most 1536 */
     TC_PREC_MIXED = 1,      /* FFTs, products and explicit radial rows in
                                float32, their continuity term in double-float;
                                banded solves, RK memory, reconstruction and
                                the mean mode in float64 */
-    TC_PREC_DF64 = 2        /* FFTs, products and explicit radial rows in
-                               double-float arithmetic (pairs of float32, ~48
-                               significand bits) on the float32 pipe; solves,
+    TC_PREC_DF64 = 2        /* explicit radial rows in double-float arithmetic
+                               (pairs of float32, ~48 significand bits) on the
+                               float32 pipe, from products rounded to it
+                               (transforms as in TC_PREC_FP64; longer ones in
+                               double-float too); solves,
                                RK memory, reconstruction and the mean mode in
                                float64 */
 };

@@ -567,6 +567,34 @@ int init_handle(tc_handle* h) {
     }
     if ((rc_ = upload(h, d.twz_f, twz_f))) return rc_;
     if ((rc_ = upload(h, d.twt_f, twt_f))) return rc_;
+    // fixed-point plane phase of the float64 and double-float forms
+    d.Mtx = fx_length(d.Mt);
+    d.Mzx = fx_length(d.Mz);
+    d.fx = d.prec != TC_PREC_MIXED && d.Mtx > 0 && d.Mzx > 0;
+    if (d.fx) {
+        (void)std::frexp(1.0 / ((double)d.Mtx * (double)d.Mzx), &d.kexp);
+        const ld kappa = ldexpl(1.0L / ((ld)d.Mtx * (ld)d.Mzx), -d.kexp);
+        if ((rc_ = upload(h, d.twx_t, fx_table(d.Mtx, 0.0L)))) return rc_;
+        if ((rc_ = upload(h, d.twx_z, fx_table(d.Mzx, kappa)))) return rc_;
+        CK(tc_fx_attributes(d.Mtx, d.Mzx));
+    } else {
+        d.Mtx = d.Mt;
+        d.Mzx = d.Mz;
+    }
+    // fixed-point plane phase of the float64 and double-float forms
+    d.Mtx = fx_length(d.Mt);
+    d.Mzx = fx_length(d.Mz);
+    d.fx = d.prec != TC_PREC_MIXED && d.Mtx > 0 && d.Mzx > 0;
+    if (d.fx) {
+        (void)std::frexp(1.0 / ((double)d.Mtx * (double)d.Mzx), &d.kexp);
+        const ld kappa = ldexpl(1.0L / ((ld)d.Mtx * (ld)d.Mzx), -d.kexp);
+        if ((rc_ = upload(h, d.twx_t, fx_table(d.Mtx, 0.0L)))) return rc_;
+        if ((rc_ = upload(h, d.twx_z, fx_table(d.Mzx, kappa)))) return rc_;
+        CK(tc_fx_attributes(d.Mtx, d.Mzx));
+    } else {
+        d.Mtx = d.Mt;
+        d.Mzx = d.Mz;
+    }
     // fields
     const size_t P1 = (size_t)d.Nr * d.npairs;
     double2* f[6];
@@ -577,11 +605,15 @@ int init_handle(tc_handle* h) {
     if ((rc_ = dalloc(h, pr, TC_NPROD * P1))) return rc_;
     CK(cudaMemset(pr, 0, TC_NPROD * P1 * sizeof(double2)));
     d.prod = pr;
-    const size_t Z1 = (size_t)d.Nr * d.Mz * d.Nh;
+    const size_t Z1 = (size_t)d.Nr * d.Mzx * d.Nh;
     double2 *zb, *pb;
     if ((rc_ = dalloc(h, zb, 3 * Z1))) return rc_;
     if ((rc_ = dalloc(h, pb, TC_NPROD * Z1))) return rc_;
     d.zbuf = zb; d.pbuf = pb;
+    if (d.fx) {
+        if ((rc_ = dalloc(h, d.zexp, 3 * (size_t)d.Nr * d.Nh))) return rc_;
+        if ((rc_ = dalloc(h, d.pexp, 3 * (size_t)d.Nr * d.Mzx))) return rc_;
+    }
     double* mean;
     if ((rc_ = dalloc(h, mean, 6 * (size_t)d.Nr))) return rc_;
     d.U = mean; d.W = mean + d.Nr; d.HU = mean + 2 * d.Nr; d.HW = mean + 3 * d.Nr; d.eprof = mean + 4 * d.Nr;
@@ -877,13 +909,15 @@ int validate(const tc_params* p) {
 // tc_get_field and a per-allocation rounding allowance of 2 MiB).
 size_t estimate_device_bytes(const tc_params& p) {
     const size_t Nr = p.Nr, Nh = p.Ntheta / 2, Nz = p.Nz, Mt = 3 * (size_t)p.Ntheta / 2, Mz = 3 * Nz / 2;
-    const size_t np = Nz * Nh, P1 = Nr * np, Z1 = Nr * Mz * Nh;
+    const size_t Mzx = p.precision == TC_PREC_MIXED ? 0 : fx_length((int)Mz);
+    const size_t np = Nz * Nh, P1 = Nr * np, Z1 = Nr * (Mzx > Mz ? Mzx : Mz) * Nh;
     size_t b = 0;
     b += (6 + TC_NPROD) * P1 * sizeof(double2);                 // fields, products
     b += (3 + TC_NPROD) * Z1 * sizeof(double2);                 // zbuf, pbuf
     b += (3 + 3) * Nr * 5 * np * sizeof(double);                // LU tables
     b += Nr * 5 * np * sizeof(double) + 4 * Nr * np * sizeof(double);   // L band, c, c1 (+ double-float copies)
     b += Nr * Mz * Mt * sizeof(double);                         // physical output (on demand)
+    b += 3 * Nr * (Nh + Mzx) * sizeof(int);                     // exponents of the fixed-point planes
     b += 64 * Nr * sizeof(double) + 4 * (Mz + 2 * Mt) * sizeof(double2);  // radial tables, twiddles
     return b + 40 * (2u << 20);
 }

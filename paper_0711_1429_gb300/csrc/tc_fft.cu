@@ -13,6 +13,32 @@ cudaError_t tc_plane_attributes_f64();
 cudaError_t tc_plane_attributes_f32();
 cudaError_t tc_plane_attributes_df();
 cudaError_t tc_rows_phys_attributes();
+#define FX_GROUP(TAG)                                                                                                   \
+    bool tc_fx_z_##TAG(const TcDev&, const TcDev*, const int2*, int, int, cudaStream_t, int, int);                      \
+    bool tc_fx_rows_##TAG(const TcDev&, const TcDev*, const int2*, int, cudaStream_t);                                  \
+    bool tc_fx_attributes_##TAG(int, int, cudaError_t&);
+FX_GROUP(a) FX_GROUP(b) FX_GROUP(c) FX_GROUP(d)
+#undef FX_GROUP
+
+void tc_fx_plane_kernel(const TcDev& d, const TcDev* ds, const int2* ymap, int nplanes, int which, cudaStream_t s,
+                        int col0, int ncols) {
+    if (which == 1) {
+        (void)(tc_fx_rows_a(d, ds, ymap, nplanes, s) || tc_fx_rows_b(d, ds, ymap, nplanes, s) ||
+               tc_fx_rows_c(d, ds, ymap, nplanes, s) || tc_fx_rows_d(d, ds, ymap, nplanes, s));
+    } else {
+        (void)(tc_fx_z_a(d, ds, ymap, nplanes, which, s, col0, ncols) || tc_fx_z_b(d, ds, ymap, nplanes, which, s, col0, ncols) ||
+               tc_fx_z_c(d, ds, ymap, nplanes, which, s, col0, ncols) || tc_fx_z_d(d, ds, ymap, nplanes, which, s, col0, ncols));
+    }
+}
+
+cudaError_t tc_fx_attributes(int Mtx, int Mzx) {
+    cudaError_t e = cudaSuccess;
+    tc_fx_attributes_a(Mtx, Mzx, e);
+    tc_fx_attributes_b(Mtx, Mzx, e);
+    tc_fx_attributes_c(Mtx, Mzx, e);
+    tc_fx_attributes_d(Mtx, Mzx, e);
+    return e;
+}
 
 bool tc_fft_fixed_length(int M) {
     for (int m : {12, 18, 24, 36, 48, 72, 96, 144, 192, 288, 384, 576, 768, 1152, 1536})
@@ -42,14 +68,16 @@ __global__ void __launch_bounds__(256) k_energy(TcDev d) {
 }
 
 void tc_launch_plane_kernel_tiles(const TcDev& d, int which, cudaStream_t s, int tile0, int ntiles) {
-    if (d.prec == 1) tc_plane_kernel_f32(d, which, s, tile0, ntiles);
+    if (d.fx) tc_fx_plane_kernel(d, nullptr, nullptr, d.Nr, which, s, tile0 * d.ztile, ntiles * d.ztile);
+    else if (d.prec == 1) tc_plane_kernel_f32(d, which, s, tile0, ntiles);
     else if (d.prec == 2) tc_plane_kernel_df(d, which, s, tile0, ntiles);
     else tc_plane_kernel_f64(d, which, s, tile0, ntiles);
 }
 
 void tc_launch_plane_kernel_batch(const TcDev& d0, const TcDev* ds, const int2* ymap, int nplanes, int which,
                                   cudaStream_t s) {
-    if (d0.prec == 1) tc_plane_kernel_batch_f32(d0, ds, ymap, nplanes, which, s);
+    if (d0.fx) tc_fx_plane_kernel(d0, ds, ymap, nplanes, which, s, 0, d0.Nh);
+    else if (d0.prec == 1) tc_plane_kernel_batch_f32(d0, ds, ymap, nplanes, which, s);
     else if (d0.prec == 2) tc_plane_kernel_batch_df(d0, ds, ymap, nplanes, which, s);
     else tc_plane_kernel_batch_f64(d0, ds, ymap, nplanes, which, s);
 }

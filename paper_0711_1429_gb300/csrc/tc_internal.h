@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <cstddef>
 #include <cstdint>
+#include "tc_fx.cuh"
+#include "tc_fx.cuh"
 
 #define TC_MAX_STAGES 16
 #define TC_NPROD 5   // transformed products: uu-vv, uv, uw, vw, ww-vv
@@ -128,6 +130,28 @@ struct TcDev {
     const float4* twh_x;
     const float4* twr_x;
 
+    // fixed-point plane phase of the float64 and double-float forms (fx = 1
+    // where both padded lengths have a planned length at least as long):
+    // transform lengths Mtx >= Mt, Mzx >= Mz (any length from 3N/2 up keeps
+    // the quadratic products free of aliasing), tables, and the exponent of
+    // 1/(Mtx Mzx), whose mantissa is in the axial table.  fx = 0: Mtx = Mt,
+    // Mzx = Mz.
+    int fx, Mtx, Mzx, kexp;
+    const fxw* twx_t;
+    const fxw* twx_z;
+    int* zexp;                  // [3][Nr][Nh]: exponents of zbuf's columns
+    int* pexp;                  // [3][Nr][Mzx]: exponents of pbuf's rows (products 0 and 1, 2 and 3, 4)
+
+    // fixed-point plane phase of the float64 and double-float forms (fx = 1
+    // where both padded lengths have a planned length at least as long):
+    // transform lengths Mtx >= Mt, Mzx >= Mz (any length from 3N/2 up keeps
+    // the quadratic products free of aliasing), tables, and the exponent of
+    // 1/(Mtx Mzx), whose mantissa is in the axial table.  fx = 0: Mtx = Mt,
+    // Mzx = Mz.
+    int fx, Mtx, Mzx, kexp;
+    const fxw* twx_t;
+    const fxw* twx_z;
+
     // physical output buffer for tc_get_field (float64 [Nr][Mz][Mt])
     double* phys;
     // energy and strain-rate reduction outputs [Nr]
@@ -148,6 +172,14 @@ void tc_launch_plane_kernel_tiles(const TcDev& d, int which, cudaStream_t s, int
 // case; (case, radial plane) per grid row, nplanes rows)
 void tc_launch_plane_kernel_batch(const TcDev& d0, const TcDev* ds, const int2* ymap, int nplanes, int which,
                                   cudaStream_t s);
+// the fixed-point kernels (fx = 1), and their shared-memory opt-in
+void tc_fx_plane_kernel(const TcDev& d, const TcDev* ds, const int2* ymap, int nplanes, int which, cudaStream_t s,
+                        int col0, int ncols);
+cudaError_t tc_fx_attributes(int Mtx, int Mzx);
+// the fixed-point kernels (fx = 1), and their shared-memory opt-in
+void tc_fx_plane_kernel(const TcDev& d, const TcDev* ds, const int2* ymap, int nplanes, int which, cudaStream_t s,
+                        int col0, int ncols);
+cudaError_t tc_fx_attributes(int Mtx, int Mzx);
 cudaError_t tc_probe_fma(double* fp64_tflops, double* fp32_tflops);
 void tc_launch_line_phase(const TcDev& d, int k, cudaStream_t s);
 // line phase of the pairs with azimuthal index j0 <= j < j0 + nj (all axial slots)

@@ -581,20 +581,6 @@ int init_handle(tc_handle* h) {
         d.Mtx = d.Mt;
         d.Mzx = d.Mz;
     }
-    // fixed-point plane phase of the float64 and double-float forms
-    d.Mtx = fx_length(d.Mt);
-    d.Mzx = fx_length(d.Mz);
-    d.fx = d.prec != TC_PREC_MIXED && d.Mtx > 0 && d.Mzx > 0;
-    if (d.fx) {
-        (void)std::frexp(1.0 / ((double)d.Mtx * (double)d.Mzx), &d.kexp);
-        const ld kappa = ldexpl(1.0L / ((ld)d.Mtx * (ld)d.Mzx), -d.kexp);
-        if ((rc_ = upload(h, d.twx_t, fx_table(d.Mtx, 0.0L)))) return rc_;
-        if ((rc_ = upload(h, d.twx_z, fx_table(d.Mzx, kappa)))) return rc_;
-        CK(tc_fx_attributes(d.Mtx, d.Mzx));
-    } else {
-        d.Mtx = d.Mt;
-        d.Mzx = d.Mz;
-    }
     // fields
     const size_t P1 = (size_t)d.Nr * d.npairs;
     double2* f[6];

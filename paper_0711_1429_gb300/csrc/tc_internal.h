@@ -4,7 +4,6 @@
 #include <cstddef>
 #include <cstdint>
 #include "tc_fx.cuh"
-#include "tc_fx.cuh"
 
 #define TC_MAX_STAGES 16
 #define TC_NPROD 5   // transformed products: uu-vv, uv, uw, vw, ww-vv
@@ -142,16 +141,6 @@ struct TcDev {
     int* zexp;                  // [3][Nr][Nh]: exponents of zbuf's columns
     int* pexp;                  // [3][Nr][Mzx]: exponents of pbuf's rows (products 0 and 1, 2 and 3, 4)
 
-    // fixed-point plane phase of the float64 and double-float forms (fx = 1
-    // where both padded lengths have a planned length at least as long):
-    // transform lengths Mtx >= Mt, Mzx >= Mz (any length from 3N/2 up keeps
-    // the quadratic products free of aliasing), tables, and the exponent of
-    // 1/(Mtx Mzx), whose mantissa is in the axial table.  fx = 0: Mtx = Mt,
-    // Mzx = Mz.
-    int fx, Mtx, Mzx, kexp;
-    const fxw* twx_t;
-    const fxw* twx_z;
-
     // physical output buffer for tc_get_field (float64 [Nr][Mz][Mt])
     double* phys;
     // energy and strain-rate reduction outputs [Nr]
@@ -172,10 +161,6 @@ void tc_launch_plane_kernel_tiles(const TcDev& d, int which, cudaStream_t s, int
 // case; (case, radial plane) per grid row, nplanes rows)
 void tc_launch_plane_kernel_batch(const TcDev& d0, const TcDev* ds, const int2* ymap, int nplanes, int which,
                                   cudaStream_t s);
-// the fixed-point kernels (fx = 1), and their shared-memory opt-in
-void tc_fx_plane_kernel(const TcDev& d, const TcDev* ds, const int2* ymap, int nplanes, int which, cudaStream_t s,
-                        int col0, int ncols);
-cudaError_t tc_fx_attributes(int Mtx, int Mzx);
 // the fixed-point kernels (fx = 1), and their shared-memory opt-in
 void tc_fx_plane_kernel(const TcDev& d, const TcDev* ds, const int2* ymap, int nplanes, int which, cudaStream_t s,
                         int col0, int ncols);

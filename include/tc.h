@@ -94,7 +94,7 @@ typedef struct {
     int precision;          /* TC_PREC_FP64, TC_PREC_MIXED or TC_PREC_DF64     */
     int device;             /* CUDA device ordinal; < 0: current device        */
     int autotune;           /* 1: time the candidate tile shapes of the z
-                               transforms and the line-kernel variants at
+                               transforms and the line-phase variants at
                                creation, and the column groups of the step
                                graph (1 or 2) on the first tc_step of three or
                                more steps, keeping the fastest (cached per
@@ -209,31 +209,29 @@ int tc_set_stream(tc_handle* h, void* cuda_stream);
  * every choice):
  *   ztile: azimuthal columns per block of the z transforms, 1, 2, 4 or 8,
  *          dividing Ntheta/2 (0 keeps the current value);
- *   line_variant: line-kernel launch shape, 64, 128 or 256 threads per
- *          block, 1003 / 1004 (128 threads, budget for 3 / 4 blocks per
- *          SM), 2007 (64 threads, 144 registers) or 3001 (64 threads per 32
- *          pairs: one warp advances v, the other eta, for short line phases
- *          of few pairs); 0 keeps the current;
+ *   line_variant: radial rows per warp of the explicit-row kernel of the line
+ *          phase: 128 lets the library choose from the shape; 64, 256, 1003,
+ *          1004, 2007 and 3001 pin 8, 64, 16, 32, 4 and 128 rows; 0 keeps the
+ *          current;
  *   chunks: column groups of the step graph, in which the z transforms of
- *          one group overlap the line kernel of another: 1 (no overlap), 2,
+ *          one group overlap the line phase of another: 1 (no overlap), 2,
  *          4 or 8, used when it divides the number of z tiles (0 keeps the
  *          current choice, initially made from the shape).
  * Returns TC_ERR_ARG for other values; a captured step graph is rebuilt. */
 int tc_set_tiles(tc_handle* h, int ztile, int line_variant, int chunks);
 
-/* The launch shapes in use (after the autotuner): z tile, line-kernel
+/* The launch shapes in use (after the autotuner): z tile, line-phase
  * variant and column groups of the step graph (1: no overlap).  Any pointer
  * may be NULL.  A step graph launches 15 kernels without groups and
- * 7 + 8 * chunks with them, 3 more with the deferred RK memory below. */
+ * 4 + 11 * chunks with them, 3 more with the deferred RK memory below. */
 int tc_get_tiles(const tc_handle* h, int* ztile, int* line_variant, int* chunks);
 
 /* Deferred RK memory (double-float and mixed forms; no counterpart in the
  * paper, same bits either way).  The implicit part of the next substep's
  * low-storage RK memory, H += (beta_k + alpha_k+1) dt L x^(k+1) (Sec. 2.3;
  * L the implicit band of Eq. 6 or 7), needs only the new v and eta.  With
- * the deferral on, the line kernel leaves it out and a kernel of its own
- * adds it beside the next substep's theta rows, whose float32 or
- * double-float work leaves the float64 pipe idle; within one tc_step call
+ * the deferral on, the solves leave it out and a kernel of its own adds it
+ * beside the next substep's theta rows, whose float32 or double-float work leaves the float64 pipe idle; within one tc_step call
  * the last substep's term of a step runs beside the next step's first
  * theta rows, and the last one is completed before tc_step returns.
  *   mode: -1 chosen by timing with the autotuner (the default; off without
@@ -277,8 +275,9 @@ size_t tc_estimate_device_bytes(const tc_params* params);
  * same precision form, Ntheta and Nz make one shape class (any Nr, radius
  * ratio, Re and box).  Per substep, each of the three plane-phase kernels is
  * one launch per class covering all of its cases (the classes run as
- * concurrent graph branches), then the line kernel and the mean flow are one
- * launch each per precision form, covering all of its cases.  Cases are
+ * concurrent graph branches), then the line phase is two launches per
+ * precision form (explicit rows, solves), covering all of its cases and their
+ * mean flows.  Cases are
  * reached with tc_batch_case for tc_set_field / tc_get_field /
  * tc_torque_stats; the handle stays owned by the batch.  Results equal those
  * of the same case stepped alone, bit for bit.
@@ -306,9 +305,8 @@ void tc_batch_destroy(tc_batch* b);
  *     completes, so each case's step latency is its own.
  *   TC_SERVE_GROUPED: all admitted cases advance together, one step per
  *     graph launch of the batch's grouped kernels (one launch per plane
- *     kernel and shape class, one line-kernel and one mean-flow launch per
- *     precision form); the graph is captured again whenever the set of cases
- *     changes, which happens between steps only.  Every case's per-step
+ *     kernel and shape class, two line-phase launches per precision form);
+ *     the graph is captured again whenever the set of cases changes, which happens between steps only.  Every case's per-step
  *     latency is that of the group step.
  * Results equal those of the same case stepped alone in either mode.
  * Requests that alone exceed the budget are refused with TC_ERR_SIZE.

@@ -297,7 +297,7 @@ LINE_VARIANTS = (64, 128, 256, 1003, 1004, 2007, 3001)
 
 
 def tc_set_tiles(h, ztile=0, line_variant=0, chunks=0):
-    """Pin the z tile, the line-kernel variant (LINE_VARIANTS) and the column
+    """Pin the z tile, the line-phase variant (LINE_VARIANTS) and the column
     groups of the overlapped step; 0 keeps the current choice.  No launch
     shape changes the results."""
     return _check(lib().tc_set_tiles(h, ztile, line_variant, chunks))
@@ -313,7 +313,7 @@ def tc_get_tiles(h):
 def step_kernels(chunks, rk_deferred=False):
     """Kernels one step launches: the step graph, plus the three RK-memory
     kernels with the deferred RK memory."""
-    return (15 if chunks <= 1 else 7 + 8 * chunks) + (3 if rk_deferred else 0)
+    return (15 if chunks <= 1 else 4 + 11 * chunks) + (3 if rk_deferred else 0)
 
 
 def tc_set_rk_deferral(h, mode):

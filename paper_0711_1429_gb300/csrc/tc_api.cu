@@ -174,6 +174,47 @@ bool build_stencils(const std::vector<double>& r, HostStencils& S) {
     return true;
 }
 
+// Pentadiagonal factors (no pivoting) of the mean-flow systems d0 - beta_k dt L on
+// the unknowns 1 .. N-2, L_U = nu (l2 + d0/r^2), L_W = nu l2, the Dirichlet columns
+// moved to the right side and the one-sided rows 1, N-2 folded with their
+// neighbours; layout of TcDev::mean_lu.
+std::vector<double> mean_factors(const HostStencils& S, const std::vector<double>& rinv, double nu, double dt, const double* beta) {
+    const int N = (int)rinv.size();
+    std::vector<double> t((size_t)2 * 3 * N * 5, 0.0);
+    for (int p = 0; p < 2; ++p)
+        for (int k = 0; k < 3; ++k) {
+            double* q = &t[(size_t)(p * 3 + k) * N * 5];
+            auto row = [&](int j, double* A) {
+                for (int s = 0; s < 5; ++s) {
+                    const int i = S.start[j] + s;
+                    const double w0 = S.d0[j * 5 + s], w2 = S.l2[j * 5 + s];
+                    const double L = nu * (p == 0 ? std::fma(w0 * rinv[i], rinv[i], w2) : w2);
+                    A[s] = i == 0 || i == N - 1 ? 0.0 : std::fma(-(beta[k] * dt), L, w0);
+                }
+            };
+            double A1[5], A2[5], A3[5], AN[5];
+            row(1, A1); row(2, A2); row(N - 3, A3); row(N - 2, AN);
+            const double f = A1[4] / A2[4], g = AN[0] / A3[0];
+            q[0] = f;
+            q[(N - 1) * 5] = g;
+            double p2d = 1, p2c = 0, p2e = 0, p1d = 1, p1c = 0, p1e = 0;
+            for (int i = 1; i <= N - 2; ++i) {
+                double R[5] = {0, 0, 0, 0, 0};
+                if (i == 1) for (int s = 0; s < 3; ++s) R[2 + s] = std::fma(-f, A2[1 + s], A1[1 + s]);
+                else if (i == N - 2) for (int s = 0; s < 3; ++s) R[s] = std::fma(-g, A3[1 + s], AN[1 + s]);
+                else row(i, R);
+                const double m2 = i >= 3 ? R[0] / p2d : 0.0;
+                const double m1 = i >= 2 ? std::fma(-m2, p2c, R[1]) / p1d : 0.0;
+                const double dd = std::fma(-m1, p1c, std::fma(-m2, p2e, R[2])), c = std::fma(-m1, p1e, R[3]);
+                double* o = q + i * 5;
+                o[0] = m2; o[1] = m1; o[2] = 1.0 / dd; o[3] = c; o[4] = R[4];
+                p2d = p1d; p2c = p1c; p2e = p1e;
+                p1d = dd; p1c = c; p1e = R[4];
+            }
+        }
+    return t;
+}
+
 // Mixed-radix Stockham plans.  Family 0 (theta rows): radix-3 stages first,
 // then 4, then 2.  Family 1 (z columns): radix-3 stages, then 16, then one
 // stage of 8, 4 or 2.  Family 3 (float64 forward z): radix 4, then 2, then
@@ -328,7 +369,7 @@ void free_all(tc_handle* h) {
 }
 
 // Tile autotuner: candidate azimuthal tiles of the z kernels and block sizes
-// of the line kernel are timed on the (zero) initial state, which they leave
+// of the line phase are timed on the (zero) initial state, which they leave
 // unchanged, and the fastest pair is kept for the shape class (Nr, Ntheta,
 // Nz, precision).  The choice changes no arithmetic.
 std::mutex g_tune_mu;
@@ -371,7 +412,7 @@ int autotune(tc_handle* h) {
     int best_b = d.line_block;
     for (int bs : {64, 128, 256, 1003, 1004, 2007, 3001}) {
         d.line_block = bs;
-        const float ms = timed([&] { tc_launch_line_phase(d, 0, h->stream); });
+        const float ms = timed([&] { tc_launch_line_phase(d, 0, h->stream, false); });
         if (ms < best) { best = ms; best_b = bs; }
     }
     d.line_block = best_b;
@@ -379,6 +420,8 @@ int autotune(tc_handle* h) {
     cudaEventDestroy(b);
     CK(cudaGetLastError());
     CK(cudaMemset(d.flag, 0, 4 * sizeof(int)));
+    for (double2* f : {d.v, d.eta, d.u, d.w, d.Hv, d.He})
+        CK(cudaMemset(f, 0, (size_t)d.Nr * d.npairs * sizeof(double2)));
     std::lock_guard<std::mutex> lk(g_tune_mu);
     g_tune[key] = {d.ztile, d.line_block};
     return TC_OK;
@@ -472,6 +515,12 @@ int init_handle(tc_handle* h) {
         if ((rc_ = upload(h, d.l1x, dsplit(h->S.l1)))) return rc_;
         if ((rc_ = upload(h, d.l2x, dsplit(h->S.l2)))) return rc_;
         if ((rc_ = upload(h, d.rinvx, dsplit(rinv)))) return rc_;
+        std::vector<double> l1e(h->S.l1);
+        for (int j = 1; j < P.Nr - 1; ++j)
+            for (int s = 0; s < 5; ++s) l1e[j * 5 + s] += 2.0 * h->S.d0[j * 5 + s] * rinv[h->S.start[j] + s];
+        if ((rc_ = upload(h, d.l1e, l1e))) return rc_;
+        if ((rc_ = upload(h, d.l1ex, dsplit(l1e)))) return rc_;
+        if ((rc_ = upload(h, d.mean_lu, mean_factors(h->S, rinv, d.nu, d.dt, d.rk_beta)))) return rc_;
     }
     // FFT plans
     std::vector<ld> zr, zi, tr, ti, hr, hi;
@@ -618,6 +667,7 @@ int init_handle(tc_handle* h) {
     if ((rc_ = dalloc(h, d.tab_luv, 3 * (size_t)d.Nr * 5 * d.npairs))) return rc_;
     if ((rc_ = dalloc(h, d.tab_lue, 3 * (size_t)d.Nr * 5 * d.npairs))) return rc_;
     if ((rc_ = dalloc(h, d.tab_lv, (size_t)d.Nr * 5 * d.npairs))) return rc_;
+    if ((rc_ = dalloc(h, d.tab_le, (size_t)d.Nr * 5 * d.npairs))) return rc_;
     if ((rc_ = dalloc(h, d.tab_c, (size_t)d.Nr * d.npairs))) return rc_;
     if ((rc_ = dalloc(h, d.tab_c1, (size_t)d.Nr * d.npairs))) return rc_;
     if (d.prec != TC_PREC_FP64) {     // float (hi, lo) copies of c and c'
@@ -636,6 +686,9 @@ int init_handle(tc_handle* h) {
     CK(cudaMemcpy(hf, d.flag, sizeof(hf), cudaMemcpyDeviceToHost));
     if (hf[1]) { set_err("a radial system has a vanishing pivot (LU without pivoting)"); return TC_ERR_STATE; }
     if (P.autotune) {
+        // the timed kernels read the plane buffers
+        CK(cudaMemset(d.pbuf, 0, TC_NPROD * Z1 * sizeof(double2)));
+        if (d.fx) CK(cudaMemset(d.pexp, 0, 3 * (size_t)d.Nr * d.Mzx * sizeof(int)));
         if ((rc_ = autotune(h))) return rc_;
     }
     h->need_init = true;
@@ -664,7 +717,6 @@ int prepare_pipeline(tc_handle* h) {
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->evz[c], cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->evl[c], cudaEventDisableTiming);
     }
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->evm, cudaEventDisableTiming);
     for (auto& ev : h->evj)
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->srk, cudaStreamNonBlocking);
@@ -687,8 +739,6 @@ void release_pipeline(tc_handle* h) {
         if (h->evl[c]) cudaEventDestroy(h->evl[c]);
         h->evz[c] = h->evl[c] = nullptr;
     }
-    if (h->evm) cudaEventDestroy(h->evm);
-    h->evm = nullptr;
     for (auto& ev : h->evj) { if (ev) cudaEventDestroy(ev); ev = nullptr; }
     if (h->srk) cudaStreamDestroy(h->srk);
     if (h->evrk0) cudaEventDestroy(h->evrk0);
@@ -712,18 +762,18 @@ int pipeline_chunks(const tc_handle* h) {
 
 // One step.  Without column groups: the 15 kernels in order.  With C groups
 // the plane and line phases overlap: the z-forward transform of group c is
-// followed at once by the line kernel of group c (its pairs need only that
+// followed at once by the line phase of group c (its pairs need only that
 // group's products), whose output feeds the next substep's z-inverse
-// transform of group c; the mean flow needs the j = 0 column (group 0) and
-// must precede the z inverse of group 0 (its (0,0) slot holds U, W).  The
-// theta rows of each substep wait for every group.  The line kernels of
+// transform of group c; the mean flow goes with group 0, whose column j = 0
+// holds its products and, for the z inverse, U and W.  The
+// theta rows of each substep wait for every group.  The line phases of
 // alternate groups use two streams so that they overlap too.
 // Deferred RK memory (double-float and mixed forms, inside a captured step):
-// the line kernels leave out the implicit part of the next RK memory, and
+// the solves leave out the implicit part of the next RK memory, and
 // k_rk_memory adds it for substep k - 1 on its own stream beside the theta
 // rows of substep k, whose float32 work leaves the float64 pipe idle; the
-// line kernel of substep k waits for it.  The last substep's memory is
-// completed at the end of the step.  Same bits as the full line kernel.
+// line phase of substep k waits for it.  The last substep's memory is
+// completed at the end of the step.  Same bits as the full solves.
 bool defer_rk(const tc_handle* h) {
     const int m = h->rk_defer >= 0 ? h->rk_defer : h->rk_defer_auto;
     return h->pipe_ready && h->d.prec != TC_PREC_FP64 && m == 1;
@@ -741,8 +791,7 @@ static void rk_fork(tc_handle* h, int kprev, cudaStream_t s) {
     cudaEventRecord(h->evrk1, h->srk);
 }
 static void line_chunk(const tc_handle* h, int k, cudaStream_t s, int ja, int jw) {
-    if (defer_rk(h)) tc_launch_line_chunk_deferred(h->d, k, s, ja, jw);
-    else tc_launch_line_chunk(h->d, k, s, ja, jw);
+    tc_launch_line_chunk(h->d, k, s, ja, jw, ja == 0, defer_rk(h));
 }
 
 // With the deferred RK memory, `lead` starts the step with the previous
@@ -754,34 +803,20 @@ void launch_step(tc_handle* h, cudaStream_t s, bool lead, bool trail) {
     const bool defer = defer_rk(h);
     auto pending = [&](int k) { return defer && (k > 0 || lead); };   // an RK memory to add before line k
     if (C <= 1) {
-        // the mean flow (one block) runs beside the line kernel, which does
-        // not touch U, W or the (0,0) slot; the next z inverse waits for it
-        const bool side = h->pipe_ready;
         for (int k = 0; k < 3; ++k) {
-            if (side && k > 0) cudaStreamWaitEvent(s, h->evm, 0);
             tc_launch_plane_kernel(d, 0, s);
             if (pending(k)) rk_fork(h, k > 0 ? k - 1 : 2, s);
             tc_launch_plane_kernel(d, 1, s);
             tc_launch_plane_kernel(d, 2, s);
             if (pending(k)) cudaStreamWaitEvent(s, h->evrk1, 0);
-            if (side) {
-                cudaEventRecord(h->evz[0], s);
-                cudaStreamWaitEvent(h->aux[2], h->evz[0], 0);
-                tc_launch_mean_phase(d, k, h->aux[2]);
-                cudaEventRecord(h->evm, h->aux[2]);
-                line_chunk(h, k, s, 0, d.Nh);
-            } else {
-                line_chunk(h, k, s, 0, d.Nh);
-                tc_launch_mean_phase(d, k, s);
-            }
+            line_chunk(h, k, s, 0, d.Nh);
         }
-        if (side) cudaStreamWaitEvent(s, h->evm, 0);
         if (defer && trail) tc_launch_rk_memory(d, 2, s, 0, d.Nh, false);
         return;
     }
     const int tpc = (d.Nh / d.ztile) / C;      // z tiles per group
     const int cw = tpc * d.ztile;              // columns per group
-    cudaStream_t sM = h->aux[2], sZ = h->aux[3];
+    cudaStream_t sZ = h->aux[2];
     tc_launch_plane_kernel(d, 0, s);           // z inverse of the first substep
     for (int k = 0; k < 3; ++k) {
         if (pending(k)) rk_fork(h, k > 0 ? k - 1 : 2, s);
@@ -790,9 +825,6 @@ void launch_step(tc_handle* h, cudaStream_t s, bool lead, bool trail) {
             tc_launch_plane_kernel_tiles(d, 2, s, c * tpc, tpc);
             cudaEventRecord(h->evz[c], s);
         }
-        cudaStreamWaitEvent(sM, h->evz[0], 0);
-        tc_launch_mean_phase(d, k, sM);
-        cudaEventRecord(h->evm, sM);
         for (int c = 0; c < C; ++c) {
             cudaStream_t sL = h->aux[c & 1];
             cudaStreamWaitEvent(sL, h->evz[c], 0);
@@ -801,11 +833,10 @@ void launch_step(tc_handle* h, cudaStream_t s, bool lead, bool trail) {
             cudaEventRecord(h->evl[c], sL);
             if (k < 2) {
                 cudaStreamWaitEvent(sZ, h->evl[c], 0);
-                if (c == 0) cudaStreamWaitEvent(sZ, h->evm, 0);
                 tc_launch_plane_kernel_tiles(d, 0, sZ, c * tpc, tpc);
             }
         }
-        for (int a = 0; a < (k < 2 ? 4 : 3); ++a) {
+        for (int a = 0; a < (k < 2 ? 3 : 2); ++a) {
             cudaEventRecord(h->evj[a], h->aux[a]);
             cudaStreamWaitEvent(s, h->evj[a], 0);
         }
@@ -901,7 +932,7 @@ size_t estimate_device_bytes(const tc_params& p) {
     b += (6 + TC_NPROD) * P1 * sizeof(double2);                 // fields, products
     b += (3 + TC_NPROD) * Z1 * sizeof(double2);                 // zbuf, pbuf
     b += (3 + 3) * Nr * 5 * np * sizeof(double);                // LU tables
-    b += Nr * 5 * np * sizeof(double) + 4 * Nr * np * sizeof(double);   // L band, c, c1 (+ double-float copies)
+    b += 2 * Nr * 5 * np * sizeof(double) + 4 * Nr * np * sizeof(double);   // L bands, c, c1 (+ double-float copies)
     b += Nr * Mz * Mt * sizeof(double);                         // physical output (on demand)
     b += 3 * Nr * (Nh + Mzx) * sizeof(int);                     // exponents of the fixed-point planes
     b += 64 * Nr * sizeof(double) + 4 * (Mz + 2 * Mt) * sizeof(double2);  // radial tables, twiddles
@@ -1025,7 +1056,7 @@ namespace {
 // With the autotuner on, the first tc_step of three or more steps runs one
 // self-contained step with each candidate launch plan not pinned by the
 // caller: 1 and 2 column groups and, in the double-float and mixed forms,
-// the RK memory's implicit part in the line kernel or deferred beside the
+// the RK memory's implicit part in the solves or deferred beside the
 // theta rows.  Each is timed with events; the fastest is kept for this
 // handle and the shape class.  Every plan gives the same bits, so the tuning
 // steps are ordinary steps.
@@ -1112,8 +1143,7 @@ int tc_advance_substeps(tc_handle* h, int nsub) {
     for (int n = 0; n < nsub; ++n) {
         const int k = h->phase;
         tc_launch_plane_phase(h->d, h->stream);
-        tc_launch_line_phase(h->d, k, h->stream);
-        tc_launch_mean_phase(h->d, k, h->stream);
+        tc_launch_line_phase(h->d, k, h->stream, true);
         CK(cudaGetLastError());
         h->phase = (k + 1) % 3;
         if (h->phase == 0) { h->t += h->d.dt; h->step += 1; }
@@ -1165,8 +1195,7 @@ int tc_split_pairs(tc_handle* h) {
     int rc;
     if ((rc = ensure_init(h))) return rc;
     const int k = h->phase;
-    tc_launch_line_chunk(h->d, k, h->stream, h->split_j0, h->split_j1 - h->split_j0);
-    if (h->split_j0 == 0) tc_launch_mean_phase(h->d, k, h->stream);
+    tc_launch_line_chunk(h->d, k, h->stream, h->split_j0, h->split_j1 - h->split_j0, h->split_j0 == 0, false);
     CK(cudaGetLastError());
     h->phase = (k + 1) % 3;
     if (h->phase == 0) { h->t += h->d.dt; h->step += 1; }
@@ -1470,7 +1499,7 @@ int tc_phase_times(tc_handle* h, int nsteps, double* ms, int nphases) {
                 tc_launch_plane_kernel(h->d, w, h->stream);
                 CK(cudaEventRecord(ev[w + 1], h->stream));
             }
-            tc_launch_line_phase(h->d, k, h->stream);
+            tc_launch_line_phase(h->d, k, h->stream, false);
             CK(cudaEventRecord(ev[4], h->stream));
             tc_launch_mean_phase(h->d, k, h->stream);
             CK(cudaEventRecord(ev[5], h->stream));

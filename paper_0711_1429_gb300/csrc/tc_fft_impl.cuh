@@ -959,7 +959,7 @@ __device__ __forceinline__ void zfwd_body(const TcDev& d, int tile0, int bx, int
     else if constexpr (std::is_same<T, float>::value) scale = d.fscale_f;
     else scale = dfloat(d.fscale_f, d.fscale_lo);
     // products: double2 for float64, float2 for the mixed form, double-float
-    // pairs for the double-float form (read as such by the line kernel)
+    // pairs for the double-float form (read as such by the explicit rows)
     typedef typename std::conditional<std::is_same<T, double>::value, double2, C>::type PO;
     PO* outp = reinterpret_cast<PO*>(d.prod) + ((size_t)p * Nr + r) * Nz * Nh;
     for (int idx = threadIdx.x; idx < ct * Nz; idx += blockDim.x) {

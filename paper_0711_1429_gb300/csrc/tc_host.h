@@ -33,13 +33,13 @@ struct tc_handle {
     cudaStream_t own_stream = nullptr;   // created by the batch / server
     // overlap of the plane and line phases inside a captured step: the
     // azimuthal columns are split into `chunks` groups of z tiles; aux
-    // streams 0, 1 run the line kernel of alternate chunks, 2 the mean flow,
-    // 3 the next substep's z inverse (0 chunks: chosen from the shape)
+    // streams 0, 1 run the line phase of alternate chunks, 2 the next substep's
+    // z inverse (0 chunks: chosen from the shape)
     int chunks = 0;                // set by tc_set_tiles (0: automatic)
     int chunks_auto = 0;           // chosen by timing the first steps (0: not yet)
     bool pipe_ready = false;
-    cudaStream_t aux[4] = {nullptr, nullptr, nullptr, nullptr};
-    cudaEvent_t evz[TC_MAX_CHUNKS] = {}, evl[TC_MAX_CHUNKS] = {}, evm = nullptr, evj[4] = {};
+    cudaStream_t aux[3] = {nullptr, nullptr, nullptr};
+    cudaEvent_t evz[TC_MAX_CHUNKS] = {}, evl[TC_MAX_CHUNKS] = {}, evj[3] = {};
     // deferred RK memory (double-float and mixed forms): the implicit part of
     // substep k's RK memory runs on srk beside the theta rows of substep k+1
     // (rk_defer: -1 chosen by timing, 0 off, 1 on; rk_defer_auto: the

@@ -44,8 +44,7 @@ struct TcDev {
     int mixed;                  // 1: float32 FFT/products (precision == TC_PREC_MIXED)
     int prec;                   // TC_PREC_FP64, TC_PREC_MIXED or TC_PREC_DF64
     int ztile;                  // azimuthal columns per CTA of the z kernels (divides Nh)
-    int line_block;             // line-kernel variant: 64/128/256 threads, or 1003/1004 =
-                                // 128 threads with registers for 3/4 resident blocks per SM
+    int line_block;             // radial rows per warp of k_explicit (explicit_rows_per_warp)
     double dt, nu, m0, alpha0, W_outer;
     double fscale;              // 1/(Mt Mz), the forward-transform factor
     float fscale_f;
@@ -84,12 +83,17 @@ struct TcDev {
     const float2* l1x;
     const float2* l2x;
     const float2* rinvx;
-    const double* mean_lu;      // [2 profiles][3 substeps][Nr][5] + precombination
-    const double* mean_L;       // [2][Nr][5] implicit bands of U and W rows
+    const double* l1e;          // l1 + 2 d0/r: stencil of the eta rows' B term (k_explicit)
+    const float2* l1ex;         // its double-float copy
+    // factors of the mean-flow systems [U, W][3 substeps][Nr][5]: (m2, m1, 1/diag,
+    // c, e) per row; entry 0 of rows 0 and Nr - 1: the factors that fold the
+    // one-sided rows 1 and Nr - 2 with their neighbours
+    const double* mean_lu;
     // per-pair tables, structure of arrays [..][Nr][5][npairs]
     double* tab_luv;            // [3][Nr][5][npairs]
     double* tab_lue;            // [3][Nr][5][npairs]
-    double* tab_lv;             // [Nr][5][npairs]
+    double* tab_lv;             // [Nr][5][npairs] implicit bands of the v rows and of the eta rows over nu
+    double* tab_le;
     double* tab_c;              // [Nr][npairs] c = 1/k^2
     double* tab_c1;             // [Nr][npairs] c1 = dc/dr
     float2* tab_cx;             // double-float copies of c, c1 (TC_PREC_DF64 only)
@@ -166,24 +170,28 @@ void tc_fx_plane_kernel(const TcDev& d, const TcDev* ds, const int2* ymap, int n
                         int col0, int ncols);
 cudaError_t tc_fx_attributes(int Mtx, int Mzx);
 cudaError_t tc_probe_fma(double* fp64_tflops, double* fp32_tflops);
-void tc_launch_line_phase(const TcDev& d, int k, cudaStream_t s);
-// line phase of the pairs with azimuthal index j0 <= j < j0 + nj (all axial slots)
-void tc_launch_line_chunk(const TcDev& d, int k, cudaStream_t s, int j0, int nj);
-// the same without the implicit part of the next RK memory (double-float and
-// mixed forms; float64 launches the full kernel), which tc_launch_rk_memory
-// then adds for the same pairs before the next substep's line kernel
-void tc_launch_line_chunk_deferred(const TcDev& d, int k, cudaStream_t s, int j0, int nj);
+// line phase of all pairs, and of the pairs with azimuthal index j0 <= j < j0 + nj
+// (all axial slots).  mean: with the mean flow (once per substep).  deferred:
+// without the implicit part of the next RK memory (double-float and mixed forms;
+// float64 keeps it), which tc_launch_rk_memory then adds for the same pairs
+// before the next substep's line phase
+void tc_launch_line_phase(const TcDev& d, int k, cudaStream_t s, bool mean);
+void tc_launch_line_chunk(const TcDev& d, int k, cudaStream_t s, int j0, int nj, bool mean, bool deferred);
 // (background: in four blocks per SM, for a launch beside other kernels)
 void tc_launch_rk_memory(const TcDev& d, int k, cudaStream_t s, int j0, int nj, bool background);
 const void* tc_rk_memory_kernel();   // its kernel, to find its nodes in a captured graph
 void tc_launch_mean_phase(const TcDev& d, int k, cudaStream_t s);
 // line phase and mean flow of substep k for many cases of one precision form
-// (descriptors ds on the device): the line kernel in nblocks blocks of
-// tc_line_batch_block() threads, bmap[block] = (case, block within the case);
-// the mean flow one block per case, maxNr the largest Nr among them
-void tc_launch_line_batch(int prec, const TcDev* ds, const int2* bmap, int nblocks, int k, cudaStream_t s);
-void tc_launch_mean_batch(int prec, const TcDev* ds, int ncases, int maxNr, int k, cudaStream_t s);
-int tc_line_batch_block();
+// (descriptors ds on the device), two launches: the explicit rows, emap[block] =
+// (case, block within the case), and the solves, bmap[block] = (case, 16 pairs of
+// the case); -1 for the block of a case is its mean flow, in the second launch if
+// `wide`, else in the first.  maxNr: the largest Nr among them, Lc: rows of a chunk
+void tc_line_batch_plan(const TcDev* ds, int ncases, int& Lc, bool& wide);
+int tc_line_batch_explicit_blocks(const TcDev& d, int Lc);
+int tc_line_batch_solve_blocks(const TcDev& d);
+void tc_launch_explicit_batch(int prec, const TcDev* ds, const int2* emap, int nblocks, int maxNr, int Lc, bool mean, int k,
+                              cudaStream_t s);
+void tc_launch_solve_batch(const TcDev* ds, const int2* bmap, int nblocks, int maxNr, bool wide, int k, cudaStream_t s);
 void tc_launch_setup_tables(const TcDev& d, cudaStream_t s);
 void tc_launch_init_state(const TcDev& d, cudaStream_t s);
 // zero the (0,0) and Nyquist slots and make the m = 0 column Hermitian

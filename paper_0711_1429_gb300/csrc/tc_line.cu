@@ -2,9 +2,8 @@
 // and Eq. 7 (eta), the banded radial solves, the Runge-Kutta memory and the
 // reconstruction of u, w from continuity; plus the mean flow (m = alpha = 0).
 //
-// One thread owns one pair and walks its radial line; the 32 threads of a
-// warp hold 32 consecutive azimuthal indices at one axial slot, so every
-// radial point is one coalesced 512-byte access per field.
+// The 32 threads of a warp hold 32 consecutive azimuthal indices at one axial
+// slot, so every radial point is one coalesced 512-byte access per field.
 //
 // Notation (Appendix): D f = f', D_* f = f' + f/r, k^2 = alpha^2 + m^2/r^2,
 // c = 1/k^2, c1..c3 its r-derivatives, nu = 2/Re.  On row j a chain operator
@@ -56,7 +55,6 @@ __device__ __forceinline__ double2 caxpy(double2 a, double s, double2 b) { retur
 __device__ __forceinline__ double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
 // finiteness from the exponent bits (integer pipe, no float64 compare)
 __device__ __forceinline__ bool dfinite(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
-__device__ __forceinline__ bool cfinite(double2 a) { return dfinite(a.x) && dfinite(a.y); }
 
 __device__ __forceinline__ double2 ld_prod(const double2* p, size_t o) { return p[o]; }
 __device__ __forceinline__ double2 ld_prod(const float2* p, size_t o) { float2 f = p[o]; return make_double2(d_bits(f.x), d_bits(f.y)); }
@@ -65,11 +63,12 @@ __device__ __forceinline__ double2 ld_prod(const float2* p, size_t o) { float2 f
 template <typename CT> __device__ __forceinline__ CT tz() { CT r; r.x = 0; r.y = 0; return r; }
 template <typename CT, typename T> __device__ __forceinline__ CT timag(T s, CT a) { CT r; r.x = -s * a.y; r.y = s * a.x; return r; }
 template <typename CT> __device__ __forceinline__ CT tadd(CT a, CT b) { CT r; r.x = a.x + b.x; r.y = a.y + b.y; return r; }
+template <typename CT> __device__ __forceinline__ CT tsub(CT a, CT b) { CT r; r.x = a.x - b.x; r.y = a.y - b.y; return r; }
 template <typename CT, typename T> __device__ __forceinline__ CT taxpy(CT a, T s, CT b) { CT r; r.x = fma(s, b.x, a.x); r.y = fma(s, b.y, a.y); return r; }
 template <typename CT, typename T> __device__ __forceinline__ CT tscale(T s, CT a) { CT r; r.x = s * a.x; r.y = s * a.y; return r; }
 __device__ __forceinline__ double2 to_d2(double2 a) { return a; }
 // float32 <-> float64 through the integer conversions of tc_dfloat.h (the
-// float64 pipe is the mixed line kernel's bottleneck); the double-float form
+// float64 pipe is the mixed line phase's bottleneck); the double-float form
 // converts with float64 instructions, which measured faster there (fewer
 // registers in a kernel that is already at its register budget)
 __device__ __forceinline__ double2 to_d2(float2 a) { return make_double2(d_bits(a.x), d_bits(a.y)); }
@@ -189,6 +188,11 @@ __device__ bool band_lu(const TcDev& d, double* tab, int k, int pair, RowFn row)
     return ok;
 }
 
+// k^2 = alpha^2 + m^2/r^2 of the implicit eta band
+__device__ __forceinline__ double k2_at(double m, double al, double ri) {
+    return __fma_rn(__dmul_rn(m, m), __dmul_rn(ri, ri), __dmul_rn(al, al));
+}
+
 // Per-pair tables: LU factors of (M - beta_k dt L) for v and eta, k = 0..2,
 // with the boundary rows folded in, and the implicit band L of the v rows.
 __global__ void __launch_bounds__(128) k_setup(TcDev d) {
@@ -217,6 +221,10 @@ __global__ void __launch_bounds__(128) k_setup(TcDev d) {
         v_band(d, j, m, al, M5, L5);
         for (int s = 0; s < 5; ++s) TAB(d.tab_lv, 0, j, s) = L5[s];
     }
+    // and of the eta rows, over nu
+    for (int j = 1; j <= N - 2; ++j)
+        for (int s = 0; s < 5; ++s)
+            TAB(d.tab_le, 0, j, s) = fma(-d.d0[j * 5 + s], k2_at(m, al, d.rinv[d.start[j] + s]), d.l2[j * 5 + s]);
     for (int k = 0; k < 3; ++k) {
         const double bdt = d.rk_beta[k] * d.dt;
         // ---- v system ----
@@ -368,14 +376,31 @@ __device__ void reconstruct_pair(const TcDev& d, int pair, double m, double al, 
 }
 
 // ---------------------------------------------------------------------------
-// One substep of the line phase, one thread per Fourier pair, for the pairs
-// of the azimuthal columns ja .. ja + jw - 1 in every axial slot (all pairs
-// when ja = 0, jw = Ntheta/2).
+// The line phase of one substep, for the pairs of the azimuthal columns
+// ja .. ja + jw - 1 in every axial slot (all pairs when ja = 0, jw = Ntheta/2):
+// two kernels.
 //
-// Explicit rows E (Eq. 6 rows 2..Nr-3, Eq. 7 rows 1..Nr-2) are sums over the
-// 5 stencil points of d0 . A + l1 . B (+ l2 . C for v), where A, B, C are
-// pointwise "inner" functions of the products and of u, v, w at that point.
-// With the five products a = uu - vv, uv, uw, vw, b = ww - vv:
+// k_explicit, one warp per 32 pairs and chunk of radial rows: the explicit rows E
+// (Eq. 6 rows 2..Nr-3, Eq. 7 rows 1..Nr-2), the right sides
+// RHS = H_k + gamma_k dt E (v: scratch, eta: in place, which no explicit row
+// reads) and H = RHS + zeta_(k+1) dt E.
+// k_solve, two warps per 16 pairs (k_solve_shared, eight, for few pairs): one warp runs the recurrences of v (the
+// banded solve and later the compact Dv solve), another those of eta; what is not
+// serial in r -- the right sides l1 . v of the Dv solve, H += (beta_k + alpha_(k+1))
+// dt L x, and u, w from continuity -- all warps share by radial rows.
+//
+// What bounds it: the float64 pipe, 64 cycles for a warp's operation on its quarter
+// of an SM, however few lanes it has.  One thread that walked a pair's whole line
+// kept a small case on the few quarters its warps filled (256 pairs: eight) and
+// put every operation of a row behind the one before; only the recurrences, an
+// eighth of the operations, are serial in r.  Per substep, line phase of the
+// float64 form before and now: 33x16x16 333 -> 45 us, 64x32x64 684 -> 82,
+// 129x128x128 1118 -> 536, 129x512x170 2897 -> 2400, 257x512x512 15.5 -> 13.5 ms; of
+// the mixed form: 129x128x128 923 -> 350 us, 257x512x512 8.7 -> 8.1 ms.
+//
+// Explicit rows: sums over the 5 stencil points of d0 . A + l1 . B (+ l2 . C for
+// v), where A, B, C are pointwise "inner" functions of the products and of u, v, w
+// at that point.  With the five products a = uu - vv, uv, uw, vw, b = ww - vv:
 //   v:   A = -i alpha uv - i m/r vw + b/r                 - 2 i nu m w/r^2
 //        B = i alpha c1 uv - i m (2c/r^2 - c1/r) vw + c alpha^2 a
 //            + 2 c alpha m/r uw + c m^2/r^2 b             - 2 i nu m c1 w/r^2
@@ -392,408 +417,740 @@ __device__ void reconstruct_pair(const TcDev& d, int pair, double m, double al, 
 // products; the right sides, the solves, the RK memory and the
 // reconstruction are float64 in every form.
 //
-// Inner functions of the explicit rows at one radial point, from the five
-// products and u, v, w: A, B, C of the v rows (C without the continuity
-// term) and A, B of the eta rows, as listed above.
-template <typename T, typename CT>
-__device__ __forceinline__ void inner_terms(const CT& pa, const CT& uv, const CT& uw, const CT& vw, const CT& pb,
-                                            const CT& U, const CT& V, const CT& W, T ri, T c, T c1,
-                                            T mt, T at, T nut, CT& a, CT& b, CT& cc, CT& ae, CT& be) {
-    const T ri2 = ri * ri;
+// Inner functions as listed above (float32 of the mixed form), C without the
+// continuity term.  Which product of a sum of two is fused is written out, so that
+// the rounding does not depend on what the compiler makes of the surrounding loop.
+__device__ __forceinline__ float sum2(float p, float x, float q, float y) { return fmaf(p, x, __fmul_rn(q, y)); }
+__device__ __forceinline__ float2 ifma(float s, float2 x, float2 acc) { return make_float2(fmaf(-s, x.y, acc.x), fmaf(s, x.x, acc.y)); }
+__device__ __forceinline__ void inner_terms(const float2& pa, const float2& uv, const float2& uw, const float2& vw, const float2& pb,
+                                            const float2& U, const float2& V, const float2& W, float ri, float c, float c1,
+                                            float mt, float at, float nut, float2& a, float2& b, float2& cc, float2& ae,
+                                            float2& be) {
+    const float ri2 = ri * ri, mr = mt * ri;
     // v rows
-    a = timag(-at, uv);
-    a = tadd(a, timag(-mt * ri, vw));
+    a = make_float2(sum2(at, uv.y, mr, vw.y), sum2(-mr, vw.x, -at, uv.x));
     a = taxpy(a, ri, pb);
-    a = tadd(a, timag((T)-2 * nut * mt * ri2, W));
-    b = timag(at * c1, uv);
-    b = tadd(b, timag(-mt * ((T)2 * c * ri2 - c1 * ri), vw));
+    a = ifma(-2.0f * nut * mt * ri2, W, a);
+    const float q1 = at * c1, q2 = -mt * sum2(2.0f * c, ri2, -c1, ri);
+    b = make_float2(sum2(-q2, vw.y, -q1, uv.y), sum2(q1, uv.x, q2, vw.x));
     b = taxpy(b, c * at * at, pa);
-    b = taxpy(b, c * (T)2 * at * mt * ri, uw);
+    b = taxpy(b, c * 2.0f * at * mt * ri, uw);
     b = taxpy(b, c * mt * mt * ri2, pb);
-    b = tadd(b, timag((T)-2 * nut * mt * c1 * ri2, W));
-    cc = timag(-at * c, uv);
-    cc = tadd(cc, timag(-mt * c * ri, vw));
-    cc = tadd(cc, timag((T)2 * nut * mt * c * ri2, W));
+    b = ifma(-2.0f * nut * mt * c1 * ri2, W, b);
+    const float q3 = -at * c, q4 = -mt * c * ri;
+    cc = make_float2(sum2(-q4, vw.y, -q3, uv.y), sum2(q3, uv.x, q4, vw.x));
+    cc = ifma(2.0f * nut * mt * c * ri2, W, cc);
     // eta rows
-    ae = tscale(mt * at * ri, pa);
-    ae = tadd(ae, timag((T)-2 * mt * ri2, uv));
-    ae = taxpy(ae, mt * mt * ri2 - at * at, uw);
+    const float q5 = mt * at * ri, q6 = -2.0f * mt * ri2;
+    ae = make_float2(sum2(q5, pa.x, -q6, uv.y), sum2(q5, pa.y, q6, uv.x));
+    ae = taxpy(ae, sum2(mt * mt, ri2, -at, at), uw);
     ae = taxpy(ae, -at * mt * ri, pb);
-    ae = tadd(ae, timag((T)2 * at * ri, vw));
-    ae = tadd(ae, timag((T)4 * nut * mt * ri2 * ri, U));
-    ae = taxpy(ae, (T)2 * nut * mt * at * ri2, V);
-    be = timag(-mt * ri, uv);
-    be = tadd(be, timag(at, vw));
-    be = tadd(be, timag((T)2 * nut * mt * ri2, U));
+    ae = ifma(2.0f * at * ri, vw, ae);
+    ae = ifma(4.0f * nut * mt * ri2 * ri, U, ae);
+    ae = taxpy(ae, 2.0f * nut * mt * at * ri2, V);
+    be = make_float2(sum2(-at, vw.y, mr, uv.y), sum2(at, vw.x, -mr, uv.x));
+    be = ifma(2.0f * nut * mt * ri2, U, be);
+}
+// The same with the continuity term, for the float64 and double-float forms, in
+// which the arithmetic is what costs: shared sums are formed once (57 float64
+// operations a point instead of 88, coefficients included).
+//   Q = alpha uv + m/r vw,  S = 2 nu m/r^2 w,  T = Q - S
+//   A = -i (Q + S) + b/r,   C = -i (c T + 3 nu c1 (alpha u + m/r w))
+//   B = i (c1 T - 2 c m/r^2 vw) + c (alpha^2 a + 2 alpha m/r uw + m^2/r^2 b)
+//   N = m/r uv - alpha vw - 2 nu m/r^2 u,  B_eta = -i N
+//   A_eta = m alpha/r (a - b) + (m^2/r^2 - alpha^2) uw + 2 nu m alpha/r^2 v + (2/r) B_eta
+// The last term of A_eta is left to the stencil of B_eta: l1e = l1 + 2 d0/r.
+template <typename T> struct IsPair { static constexpr bool value = false; };
+template <> struct IsPair<dfloat> { static constexpr bool value = true; };
+template <typename T, typename CT>
+__device__ __forceinline__ void inner_terms_shared(const CT& pa, const CT& uv, const CT& uw, const CT& vw, const CT& pb,
+                                                   const CT& U, const CT& V, const CT& W, T ri, T c, T c1, T mt, T at,
+                                                   T at2, T nu2, T nu3, CT& a, CT& b, CT& cc, CT& ae, CT& be) {
+    const T mr = mt * ri, mr2 = mr * ri, mra = mr * at, n2 = nu2 * mr2;      // nu2 = 2 nu, nu3 = 3 nu
+    const CT Q = taxpy(tscale(mr, vw), at, uv);
+    CT Tm, Tp;                                  // Q - S, Q + S
+    if constexpr (sizeof(T) == sizeof(double) && !IsPair<T>::value) { Tm = taxpy(Q, -n2, W); Tp = taxpy(Q, n2, W); }
+    else { const CT S = tscale(n2, W); Tm = tsub(Q, S); Tp = tadd(Q, S); }
+    a.x = fma(ri, pb.x, Tp.y);
+    a.y = fma(ri, pb.y, -Tp.x);
+    const CT ph = taxpy(tscale(mr, W), at, U);
+    const CT Z = taxpy(tscale(c, Tm), nu3 * c1, ph);
+    cc.x = Z.y;
+    cc.y = -Z.x;
+    const CT Y = taxpy(tscale(c1, Tm), (T)-2 * c * mr2, vw);
+    const CT R = taxpy(taxpy(tscale(at2, pa), (T)2 * mra, uw), mr * mr, pb);
+    b.x = fma(c, R.x, -Y.y);
+    b.y = fma(c, R.y, Y.x);
+    const CT N = taxpy(taxpy(tscale(mr, uv), -at, vw), -n2, U);
+    be.x = N.y;
+    be.y = -N.x;
+    ae = taxpy(taxpy(tscale(mra, tsub(pa, pb)), fma(mr, mr, -at2), uw), n2 * at, V);
 }
 
-// k^2 = alpha^2 + m^2/r^2 of the implicit eta band, rounded the same way in
-// every kernel that forms it
-__device__ __forceinline__ double k2_at(double m, double al, double ri) {
-    return __fma_rn(__dmul_rn(m, m), __dmul_rn(ri, ri), __dmul_rn(al, al));
-}
+// The radial solves and sums have real coefficients, so the real and the imaginary
+// part of a pair are two lanes of a warp: a warp instruction of the float64 pipe
+// takes 64 cycles of its quarter of the SM however many of its lanes are in use, and
+// each lane then has half the operations and registers.  Component c of a field at
+// row i is base[2 i P], base = (double*)field + 2 pair + c.
+struct RowTables { const double *d0, *l1, *dsol, *rinv; };   // the case's own, or copies in shared memory
 
 // Implicit part of the next RK memory on row jr (SMR91 low storage):
-// H_(k+1) += (beta_k + alpha_(k+1)) dt L x^(k+1), with L the v band of row jr
-// (the per-pair table) or nu (l2 - d0 k^2) of the eta row, applied to the
-// window xw / ew of x^(k+1) on the row's five stencil points (k2w: k^2 at
-// those points).  The line kernel calls it during its back substitution; the
-// deferred form (k_rk_memory) calls it after a line kernel that left it out,
-// with the same operands, so both give the same bits.
-__device__ __forceinline__ void rk_memory_row(const TcDev& d, int pair, int jr, const double2* xw, const double2* ew,
-                                              const double* k2w, double hdt, double hdtnu, bool do_v, bool do_e) {
-    const size_t o = (size_t)jr * d.npairs + pair;
-    if (do_v) {
-        double2 acc = cz();
-        for (int s = 0; s < 5; ++s) acc = caxpy(acc, TAB(d.tab_lv, 0, jr, s), xw[s]);
-        d.Hv[o] = caxpy(d.Hv[o], hdt, acc);
-    }
-    if (do_e) {
-        double2 acc = cz();
-        for (int s = 0; s < 5; ++s)
-            acc = caxpy(acc, fma(-d.d0[jr * 5 + s], k2w[s], d.l2[jr * 5 + s]), ew[s]);
-        d.He[o] = caxpy(d.He[o], hdtnu, acc);
+// H_(k+1) += (beta_k + alpha_(k+1)) dt L x^(k+1), with L the band of row jr from the
+// per-pair table, applied to the window x of x^(k+1) on the row's five stencil
+// points.  k_solve calls it after its solves; the deferred form (k_rk_memory)
+// calls it after a k_solve that left it out, with the same operands, so both give
+// the same bits.
+__device__ __forceinline__ void rk_memory_row(const TcDev& d, const double* __restrict__ tab, double* H, int pair, int jr,
+                                              const double* x, double hdt) {
+    double acc = 0.0;
+    for (int s = 0; s < 5; ++s) acc = fma(TAB(tab, 0, jr, s), x[s], acc);
+    H[2 * (size_t)jr * d.npairs] = fma(hdt, acc, H[2 * (size_t)jr * d.npairs]);
+}
+// The rows centred on i0 <= i < i1 (v: 2 .. Nr - 3; the one-sided eta rows 1 and
+// Nr - 2 with their neighbours).
+__device__ __forceinline__ void rk_memory_rows(const TcDev& d, int k, int pair, int comp, int i0, int i1) {
+    const int N = d.Nr, kn = (k + 1) % 3;
+    const size_t P2 = 2 * (size_t)d.npairs;
+    const double hdt = (d.rk_beta[k] + d.rk_alpha[kn]) * d.dt, hdtnu = hdt * d.nu;
+    const size_t o = 2 * (size_t)pair + comp;
+    const double *v = reinterpret_cast<const double*>(d.v) + o, *e = reinterpret_cast<const double*>(d.eta) + o;
+    double *Hv = reinterpret_cast<double*>(d.Hv) + o, *He = reinterpret_cast<double*>(d.He) + o;
+    i0 = i0 < 2 ? 2 : i0;
+    i1 = i1 > N - 2 ? N - 2 : i1;
+    if (i0 >= i1) return;
+    double xv[5], xe[5];
+    for (int s = 0; s < 4; ++s) { xv[s + 1] = v[(i0 - 2 + s) * P2]; xe[s + 1] = e[(i0 - 2 + s) * P2]; }
+    for (int i = i0; i < i1; ++i) {
+        for (int s = 0; s < 4; ++s) { xv[s] = xv[s + 1]; xe[s] = xe[s + 1]; }
+        xv[4] = v[(i + 2) * P2];
+        xe[4] = e[(i + 2) * P2];
+        rk_memory_row(d, d.tab_lv, Hv, pair, i, xv, hdt);
+        rk_memory_row(d, d.tab_le, He, pair, i, xe, hdtnu);
+        if (i == 2) rk_memory_row(d, d.tab_le, He, pair, 1, xe, hdtnu);
+        if (i == N - 3) rk_memory_row(d, d.tab_le, He, pair, N - 2, xe, hdtnu);
     }
 }
 
-// The sweeps of one pair (ROLE 0: v and eta; 1: v only; 2: eta only, for the
-// kernel in which one thread advances v and another eta of the same pair);
-// returns false for a thread without a pair to evolve.  The arithmetic of
-// each field is the same in every role.  With NOH the implicit part of the
-// next RK memory is left to k_rk_memory (launched after this kernel, before
-// the next substep's line kernel).
-// Roles 1 and 2 run in two warps of one block and keep step: the eta thread
-// reads v of the old state at row i while the v thread overwrites row i - 2
-// with its elimination, so a block barrier opens every iteration of the
-// forward sweep and closes the sweep.  Every thread of such a block runs the
-// same loop: a thread without a pair works on a stand-in pair (n = 0,
-// j = 1, always evolved) and stores nothing.
-template <int MODE, int ROLE, bool NOH = false>
-__device__ __forceinline__ bool line_sweeps(const TcDev& d, int k, int ja, int jw, const int idx, int& pair_out,
-                                            double& m_out, double& al_out, long long& partner_out) {
+// thread idx -> pair among the columns ja .. ja + jw - 1 of every axial slot;
+// false for a thread without a pair to evolve
+__device__ __forceinline__ bool line_pair(const TcDev& d, int ja, int jw, int idx, int& pair, double& m, double& al,
+                                          long long& partner) {
+    if (idx >= d.Nz * jw) return false;
+    pair = (idx / jw) * d.Nh + ja + idx % jw;
+    partner = -1;
+    return pair_info(d, pair, m, al, partner);
+}
+// Right sides of v between the two kernels: the last third of zbuf, free from
+// the theta rows to the next z inverse, in zbuf's own layout, so that a column
+// group's share is its own columns' (the float32 planes of the mixed form fill
+// the first half of the buffer).
+__device__ __forceinline__ double2* rhs_scratch(const TcDev& d, int pair) {
+    return reinterpret_cast<double2*>(d.zbuf) + 2 * (size_t)d.Nr * d.Mzx * d.Nh + pair;
+}
+
+// The rows' inputs on their way through shared memory: in the mixed and the
+// double-float form the arithmetic of a row (float32 pipe) is shorter than its loads
+// take, and the registers of the stencils leave no room for a row's 34 to 44 words
+// ahead of time.  Every thread copies its own words (cp.async) RING - 1 rows ahead,
+// so that no barrier is needed.  (Line phase of the mixed form, 257x512x512: 8.28 ->
+// 8.14 ms; of the double-float form, 129x512x170: 1.84 -> 1.78.)  The
+// float64 form is bound by the float64 pipe and loads into registers.
+constexpr int EXPLICIT_WARPS = 4;
+template <int MODE> struct RowRing {
+    typedef typename LineTypes<MODE>::CT CT;
+    static constexpr int RING = MODE == 1 ? 4 : MODE == 2 ? 3 : 0, NT = 32 * EXPLICIT_WARPS;
+    static constexpr int FIELDS = 5 * sizeof(CT) * NT, H = FIELDS + 48 * NT, COEF = H + 32 * NT, BYTES = COEF + 16 * NT;
+    unsigned char* base;
+    __device__ CT& prod(int q) const { return *reinterpret_cast<CT*>(base + (q * NT + threadIdx.x) * sizeof(CT)); }
+    __device__ double2& field(int q) const { return *reinterpret_cast<double2*>(base + FIELDS + (q * NT + threadIdx.x) * 16); }
+    __device__ double2& memory(int q) const { return *reinterpret_cast<double2*>(base + H + (q * NT + threadIdx.x) * 16); }
+    __device__ float2& coef(int q) const { return *reinterpret_cast<float2*>(base + COEF + (q * NT + threadIdx.x) * 8); }
+};
+template <int BYTES> __device__ __forceinline__ void copy_async(void* to, const void* from) {
+    const unsigned a = (unsigned)__cvta_generic_to_shared(to);
+    if constexpr (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(from) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(a), "l"(from) : "memory");
+}
+
+// Rows centred on c0 <= j < c1 of 2 .. Nr - 3; the one-sided eta rows 1 and
+// Nr - 2 go with their neighbours 2 and Nr - 3, whose points they use.
+template <int MODE>
+__device__ __forceinline__ void explicit_rows(const TcDev& d, int k, int ja, int jw, int idx, int c0, int c1) {
     constexpr bool MIXED = (MODE == 1);
-    constexpr bool DV = ROLE != 2, DE = ROLE != 1;
     typedef typename LineTypes<MODE>::T T;
     typedef typename LineTypes<MODE>::CT CT;
-    constexpr bool SYNC = ROLE != 0;
-    // thread idx -> pair among the columns ja .. ja + jw - 1 of every axial slot
-    bool act = idx < d.Nz * jw;
-    int pair = act ? (idx / jw) * d.Nh + ja + idx % jw : 0;
-    double m = 0.0, al = 0.0;
-    long long partner = -1;
-    if (act) act = pair_info(d, pair, m, al, partner);
-    if (!act) {
-        if constexpr (!SYNC) return false;
-        pair = 1;                                   // stand-in: loads only
-        pair_info(d, pair, m, al, partner);
-        partner = -1;
-    }
-    pair_out = pair; m_out = m; al_out = al; partner_out = partner;
+    int pair;
+    double m, al;
+    long long partner;
+    if (!line_pair(d, ja, jw, idx, pair, m, al, partner)) return;
     const int N = d.Nr;
-    const size_t P = d.npairs;
-    const CT* prod = reinterpret_cast<const CT*>(d.prod);
+    const size_t P = d.npairs, SP = (size_t)d.Mzx * d.Nh;
+    const CT* __restrict__ prod = reinterpret_cast<const CT*>(d.prod);
+    const double2* __restrict__ fu = d.u;
+    const double2* __restrict__ fv = d.v;
+    const double2* __restrict__ fw = d.w;
+    double2* rhsv = rhs_scratch(d, pair);
     const size_t PS = (size_t)N * P;            // product stride
     const int kn = (k + 1) % 3;
     const double gdt = d.rk_gamma[k] * d.dt;
     const double zdt = d.rk_zeta[kn] * d.dt;
-    const double hdt = (d.rk_beta[k] + d.rk_alpha[kn]) * d.dt;
     const double nu = d.nu;
     const T mt = (T)m, at = (T)al, nut = (T)nu;
+    const T at2 = at * at, nu2 = (T)2 * nut, nu3 = (T)3 * nut;
     // double-float constants of the mixed form's continuity term
     const dfloat mD(m), alD(al), m3nu(-3.0 * nu);
     const dfloat* l2x = reinterpret_cast<const dfloat*>(d.l2x);
     const dfloat* rinvx = reinterpret_cast<const dfloat*>(d.rinvx);
-    const T* w0s;
-    const T* w1s;
-    const T* w2s;
-    if constexpr (MODE == 1) { w0s = d.d0f; w1s = d.l1f; w2s = d.l2f; }
+    const T *w0s, *w1s, *w2s, *w1e;
+    if constexpr (MODE == 1) { w0s = d.d0f; w1s = d.l1f; w2s = d.l2f; w1e = d.l1f; }
     else if constexpr (MODE == 2) {
         w0s = reinterpret_cast<const dfloat*>(d.d0x);
         w1s = reinterpret_cast<const dfloat*>(d.l1x);
         w2s = reinterpret_cast<const dfloat*>(d.l2x);
-    } else { w0s = d.d0; w1s = d.l1; w2s = d.l2; }
+        w1e = reinterpret_cast<const dfloat*>(d.l1ex);
+    } else { w0s = d.d0; w1s = d.l1; w2s = d.l2; w1e = d.l1e; }
 
-    // ---- forward sweep: explicit rows, right sides, forward elimination ----
     CT Av[5], Bv[5], Cv[5], Ae[5], Be[5];
     dcomplex Cp[5];                             // continuity inner function (mixed form)
     for (int s = 0; s < 5; ++s) Av[s] = Bv[s] = Cv[s] = Ae[s] = Be[s] = tz<CT>();
-    double2 yv1 = cz(), yv2 = cz(), ye1 = cz(), ye2 = cz();   // y_{j-1}, y_{j-2}
-    double2 rv_prev = cz(), re_prev = cz(), re_row1 = cz();
-    const double fv = TAB(d.tab_luv, k, 0, 0), gv = TAB(d.tab_luv, k, N - 1, 0);
-    const double fe = TAB(d.tab_lue, k, 0, 0), ge = TAB(d.tab_lue, k, N - 1, 0);
-
-    auto erow = [&](int j) -> double2 {          // explicit eta row j (start = i-4)
+    auto erow = [&](int j, double2 H) {         // explicit eta row j, its right side and H
         CT acc = tz<CT>();
         for (int s = 0; s < 5; ++s) {
             acc = taxpy(acc, w0s[j * 5 + s], Ae[s]);
-            acc = taxpy(acc, w1s[j * 5 + s], Be[s]);
+            acc = taxpy(acc, w1e[j * 5 + s], Be[s]);
         }
-        return to_d2(acc);
+        const double2 E = to_d2(acc);
+        const size_t o = (size_t)j * P + pair;
+        const double2 r = caxpy(H, gdt, E);
+        d.He[o] = caxpy(r, zdt, E);
+        d.eta[o] = r;
     };
-    auto vrow = [&](int j) -> double2 {
+    auto vrow = [&](int j, double2 H) {
         CT acc = tz<CT>();
         for (int s = 0; s < 5; ++s) {
             acc = taxpy(acc, w0s[j * 5 + s], Av[s]);
             acc = taxpy(acc, w1s[j * 5 + s], Bv[s]);
             acc = taxpy(acc, w2s[j * 5 + s], Cv[s]);
         }
-        double2 r;
+        double2 E;
         if constexpr (MIXED) {
             // float32 rows plus the continuity term -3 nu l2 . (c' phi) in
             // double-float, then widened to float64
             dcomplex cc;
             for (int s = 0; s < 5; ++s) cc = dc_fma(cc, l2x[j * 5 + s], Cp[s]);
-            r = to_d2_bits(dc_fma(dc_of(acc), m3nu, cc));
+            E = to_d2_bits(dc_fma(dc_of(acc), m3nu, cc));
         } else {
-            r = to_d2(acc);
+            E = to_d2(acc);
         }
-        return r;
-    };
-    // right side of row j and the partial H_(k+1) (without the L x^k term)
-    auto rhs_v = [&](int j, double2 E) -> double2 {
         const size_t o = (size_t)j * P + pair;
-        const double2 r = caxpy(d.Hv[o], gdt, E);
-        if (act) d.Hv[o] = caxpy(r, zdt, E);
-        return r;
+        const double2 r = caxpy(H, gdt, E);
+        d.Hv[o] = caxpy(r, zdt, E);
+        rhsv[(size_t)j * SP] = r;
     };
-    auto rhs_e = [&](int j, double2 E) -> double2 {
-        const size_t o = (size_t)j * P + pair;
-        const double2 r = caxpy(d.He[o], gdt, E);
-        if (act) d.He[o] = caxpy(r, zdt, E);
-        return r;
+    typedef RowRing<MODE> Ring;
+    extern __shared__ double sm[];
+    int rd = 0, wr = 0;
+    auto fetch = [&](int i) {
+        if constexpr (Ring::RING > 0) {
+            if (i < c1 + 2) {
+                const Ring g{reinterpret_cast<unsigned char*>(sm) + wr * Ring::BYTES};
+                wr = wr + 1 == Ring::RING ? 0 : wr + 1;
+                const size_t o = (size_t)i * P + pair;
+#pragma unroll
+                for (int q = 0; q < 5; ++q) copy_async<sizeof(CT)>(&g.prod(q), prod + o + q * PS);
+                copy_async<16>(&g.field(0), fu + o);
+                copy_async<16>(&g.field(1), fv + o);
+                copy_async<16>(&g.field(2), fw + o);
+                copy_async<8>(&g.coef(0), d.tab_cx + o);
+                copy_async<8>(&g.coef(1), d.tab_c1x + o);
+                if (i >= c0 + 2) {
+                    copy_async<16>(&g.memory(0), d.Hv + o - 2 * P);
+                    copy_async<16>(&g.memory(1), d.He + o - 2 * P);
+                }
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        }
     };
-    auto fwd_v = [&](int j, double2 r) {
-        const double m2 = TAB(d.tab_luv, k, j, 0), m1 = TAB(d.tab_luv, k, j, 1);
-        const double2 y = caxpy(caxpy(r, -m2, yv2), -m1, yv1);
-        if (act) d.v[(size_t)j * P + pair] = y;
-        yv2 = yv1; yv1 = y;
-    };
-    auto fwd_e = [&](int j, double2 r) {
-        const double m2 = TAB(d.tab_lue, k, j, 0), m1 = TAB(d.tab_lue, k, j, 1);
-        const double2 y = caxpy(caxpy(r, -m2, ye2), -m1, ye1);
-        if (act) d.eta[(size_t)j * P + pair] = y;
-        ye2 = ye1; ye1 = y;
-    };
-
-    for (int i = 0; i < N; ++i) {
-        if constexpr (SYNC) __syncthreads();    // the two roles within one row of each other
+    if constexpr (Ring::RING > 0)
+        for (int q = 0; q < Ring::RING - 1; ++q) fetch(c0 - 2 + q);
+    for (int i = c0 - 2; i < c1 + 2; ++i) {
+        Ring g{reinterpret_cast<unsigned char*>(sm) + rd * Ring::BYTES};
+        if constexpr (Ring::RING > 0) {
+            fetch(i + Ring::RING - 1);
+            asm volatile("cp.async.wait_group %0;" ::"n"(Ring::RING > 0 ? Ring::RING - 1 : 0) : "memory");
+            rd = rd + 1 == Ring::RING ? 0 : rd + 1;
+        }
         for (int s = 0; s < 4; ++s) {
-            if constexpr (DV) { Av[s] = Av[s + 1]; Bv[s] = Bv[s + 1]; Cv[s] = Cv[s + 1]; Cp[s] = Cp[s + 1]; }
-            if constexpr (DE) { Ae[s] = Ae[s + 1]; Be[s] = Be[s + 1]; }
+            Av[s] = Av[s + 1]; Bv[s] = Bv[s + 1]; Cv[s] = Cv[s + 1]; Cp[s] = Cp[s + 1];
+            Ae[s] = Ae[s + 1]; Be[s] = Be[s + 1];
         }
-        {
-            const size_t o = (size_t)i * P + pair;
-            const CT pa = prod[o], uv = prod[o + PS], uw = prod[o + 2 * PS], vw = prod[o + 3 * PS], pb = prod[o + 4 * PS];
-            const double2 Ud = d.u[o], Vd = d.v[o], Wd = d.w[o];
-            const CT U = from_d2<CT>(Ud), V = from_d2<CT>(Vd), W = from_d2<CT>(Wd);
-            T ri, c, c1;
-            double c1d = 0.0;
-            if constexpr (MODE == 1) { ri = d.rinvf[i]; c = d.tab_cx[o].x; c1 = d.tab_c1x[o].x; }
-            else if constexpr (MODE == 2) { ri = as_df(d.rinvx[i]); c = as_df(d.tab_cx[o]); c1 = as_df(d.tab_c1x[o]); }
-            else { ri = d.rinv[i]; c = d.tab_c[o]; c1d = d.tab_c1[o]; c1 = c1d; }
-            CT a, b, cc, ae, be;
-            inner_terms(pa, uv, uw, vw, pb, U, V, W, ri, c, c1, mt, at, nut, a, b, cc, ae, be);
-            if constexpr (DV) {
-                if constexpr (MODE == 1) {
-                    // phi = i alpha u + (i m/r) w, times c', in double-float
-                    const dcomplex phi = dc_i(dc_fma(dc_scale(alD, dc_bits(Ud)), mD * rinvx[i], dc_bits(Wd)));
-                    Cp[4] = dc_scale(as_df(d.tab_c1x[o]), phi);
-                } else if constexpr (MODE == 2) {
-                    const CT phi = tadd(timag(at, U), timag(mt * ri, W));
-                    cc = taxpy(cc, (T)(-3.0 * nu) * c1, phi);
-                } else {
-                    const double2 phi = cadd(cimag(al, Ud), cimag(m * d.rinv[i], Wd));
-                    cc = caxpy(cc, -3.0 * nu * c1d, phi);
-                }
-                Av[4] = a; Bv[4] = b; Cv[4] = cc;
-            }
-            if constexpr (DE) { Ae[4] = ae; Be[4] = be; }
-        }
-        if (i < 4) continue;
+        const size_t o = (size_t)i * P + pair;
+        CT pa, uv, uw, vw, pb;
+        double2 Ud, Vd, Wd, Hv, He;
         const int j = i - 2;
-        if (i == 4) {
-            if constexpr (DE) re_row1 = rhs_e(1, erow(1));
-            if constexpr (DV) {
-                const double2 rv2 = rhs_v(2, vrow(2));
-                fwd_v(1, cscale(-fv, rv2));
-                fwd_v(2, rv2);
-                rv_prev = rv2;
-            }
-            if constexpr (DE) {
-                const double2 re2 = rhs_e(2, erow(2));
-                fwd_e(1, caxpy(re_row1, -fe, re2));
-                fwd_e(2, re2);
-                re_prev = re2;
-            }
-        } else if (j <= N - 3) {
-            if constexpr (DV) {
-                const double2 rv = rhs_v(j, vrow(j));
-                fwd_v(j, rv);
-                rv_prev = rv;
-            }
-            if constexpr (DE) {
-                const double2 re = rhs_e(j, erow(j));
-                fwd_e(j, re);
-                re_prev = re;
-            }
-        }
-        if (i == N - 1) {
-            if constexpr (DV) fwd_v(N - 2, cscale(-gv, rv_prev));
-            if constexpr (DE) {
-                const double2 reN = rhs_e(N - 2, erow(N - 2));
-                fwd_e(N - 2, caxpy(reN, -ge, re_prev));
-            }
-        }
-    }
-
-    if constexpr (SYNC) __syncthreads();        // the forward reads of both roles are done
-    // ---- backward sweep: back substitution, H_(k+1) += (beta+alpha') dt L x ----
-    double2 xw[5], ew[5];
-    double k2w[5];
-    for (int s = 0; s < 5; ++s) { xw[s] = cz(); ew[s] = cz(); k2w[s] = 0.0; }
-    bool bad = false;
-    if constexpr (!NOH) k2w[0] = k2_at(m, al, d.rinv[N - 1]);
-    if (act) {
-        if constexpr (DV) d.v[(size_t)(N - 1) * P + pair] = cz();
-        if constexpr (DE) d.eta[(size_t)(N - 1) * P + pair] = cz();
-    }
-    const double hdtnu = hdt * nu;
-    auto h_update = [&](int jr, bool do_v, bool do_e) {
-        if constexpr (!NOH) rk_memory_row(d, pair, jr, xw, ew, k2w, hdt, hdtnu, do_v && DV && act, do_e && DE && act);
-    };
-    for (int i = N - 2; i >= 0; --i) {
-        for (int s = 4; s > 0; --s) { xw[s] = xw[s - 1]; ew[s] = ew[s - 1]; k2w[s] = k2w[s - 1]; }
-        if constexpr (!NOH) k2w[0] = k2_at(m, al, d.rinv[i]);
-        if (i >= 1) {
-            const size_t o = (size_t)i * P + pair;
-            if constexpr (DV) {
-                const double2 yv = d.v[o];
-                const double2 xv = cscale(TAB(d.tab_luv, k, i, 2),
-                                          caxpy(caxpy(yv, -TAB(d.tab_luv, k, i, 3), xw[1]), -TAB(d.tab_luv, k, i, 4), xw[2]));
-                bad |= !cfinite(xv);
-                xw[0] = xv;
-                if (act) {
-                    d.v[o] = xv;
-                    if (partner >= 0) d.v[(size_t)i * P + partner] = cconj(xv);
-                }
-            }
-            if constexpr (DE) {
-                const double2 ye = d.eta[o];
-                const double2 xe = cscale(TAB(d.tab_lue, k, i, 2),
-                                          caxpy(caxpy(ye, -TAB(d.tab_lue, k, i, 3), ew[1]), -TAB(d.tab_lue, k, i, 4), ew[2]));
-                bad |= !cfinite(xe);
-                ew[0] = xe;
-                if (act) {
-                    d.eta[o] = xe;
-                    if (partner >= 0) d.eta[(size_t)i * P + partner] = cconj(xe);
-                }
-            }
+        if constexpr (Ring::RING > 0) {
+            pa = g.prod(0); uv = g.prod(1); uw = g.prod(2); vw = g.prod(3); pb = g.prod(4);
+            Ud = g.field(0); Vd = g.field(1); Wd = g.field(2);
+            Hv = g.memory(0); He = g.memory(1);
         } else {
-            xw[0] = cz(); ew[0] = cz();
-            if (act) {
-                if constexpr (DV) d.v[pair] = cz();
-                if constexpr (DE) d.eta[pair] = cz();
-            }
+            pa = prod[o]; uv = prod[o + PS]; uw = prod[o + 2 * PS]; vw = prod[o + 3 * PS]; pb = prod[o + 4 * PS];
+            Ud = fu[o]; Vd = fv[o]; Wd = fw[o];
         }
-        if (i == N - 5) h_update(N - 2, false, true);          // one-sided eta row N-2
-        const int jr = i + 2;
-        if (i <= N - 5 && jr >= 2) h_update(jr, true, true);
-        if (i == 0) h_update(1, false, true);                  // one-sided eta row 1
+        const CT U = from_d2<CT>(Ud), V = from_d2<CT>(Vd), W = from_d2<CT>(Wd);
+        if constexpr (MODE == 1) {
+            const float2 cx = g.coef(0), c1x = g.coef(1);
+            inner_terms(pa, uv, uw, vw, pb, U, V, W, d.rinvf[i], cx.x, c1x.x, mt, at, nut, Av[4], Bv[4], Cv[4], Ae[4], Be[4]);
+            // phi = i alpha u + (i m/r) w, times c', in double-float
+            const dcomplex phi = dc_i(dc_fma(dc_scale(alD, dc_bits(Ud)), mD * rinvx[i], dc_bits(Wd)));
+            Cp[4] = dc_scale(as_df(c1x), phi);
+        } else {
+            T ri, c, c1f;
+            if constexpr (MODE == 2) { ri = as_df(d.rinvx[i]); c = as_df(g.coef(0)); c1f = as_df(g.coef(1)); }
+            else { ri = d.rinv[i]; c = d.tab_c[o]; c1f = d.tab_c1[o]; }
+            inner_terms_shared(pa, uv, uw, vw, pb, U, V, W, ri, c, c1f, mt, at, at2, nu2, nu3, Av[4], Bv[4], Cv[4], Ae[4],
+                               Be[4]);
+        }
+        if (j < c0) continue;
+        if constexpr (Ring::RING == 0) { Hv = d.Hv[o - 2 * P]; He = d.He[o - 2 * P]; }
+        vrow(j, Hv);
+        erow(j, He);
+        if (j == 2) erow(1, d.He[P + pair]);
+        if (j == N - 3) erow(N - 2, d.He[(size_t)(N - 2) * P + pair]);
     }
-    if (bad && act) atomicOr(d.flag, 1);
-    if (act && partner >= 0) {
-        if constexpr (DV) { d.v[(size_t)(N - 1) * P + partner] = cz(); d.v[partner] = cz(); }
-        if constexpr (DE) { d.eta[(size_t)(N - 1) * P + partner] = cz(); d.eta[partner] = cz(); }
-    }
-    return act;
 }
 
-template <int MODE, bool NOH = false>
-__device__ __forceinline__ void line_body(const TcDev& d, int k, int ja, int jw, const int idx) {
-    int pair;
-    double m, al;
-    long long partner;
-    if (line_sweeps<MODE, 0, NOH>(d, k, ja, jw, idx, pair, m, al, partner)) reconstruct_pair(d, pair, m, al, partner);
+// Recurrences over n rows whose loads do not depend on them: the loads of four
+// rows stay ahead of the four rows being computed.  (A ring of eight rows, each
+// loaded as its registers come free, was slower, 13.2 -> 14.1 ms of the line phase at
+// 257x512x512: more loads in flight than a warp has scoreboards to tell apart, so that
+// waiting for a row waits for later ones.)
+template <typename D, int B = 4, typename Load, typename Step>
+__device__ __forceinline__ void rows_ahead(int n, Load load, Step step) {
+    D cur[B], nxt[B];
+#pragma unroll
+    for (int q = 0; q < B; ++q)
+        if (q < n) load(q, cur[q]);
+    for (int b = 0; b < n; b += B) {
+#pragma unroll
+        for (int q = 0; q < B; ++q)
+            if (b + B + q < n) load(b + B + q, nxt[q]);
+#pragma unroll
+        for (int q = 0; q < B; ++q)
+            if (b + q < n) step(b + q, cur[q]);
+#pragma unroll
+        for (int q = 0; q < B; ++q) cur[q] = nxt[q];
+    }
+}
+struct FwdRow { double r, m2, m1; };
+struct BackRow { double y, inv, c, e; };
+struct OneRow { double z; };
+struct MeanRow { double y, a, b, inv; };
+
+// The banded solve of one component of one field (right sides of rows 1 .. Nr - 2
+// from rhs(j)), y and then x in f (rows P2 apart), the conjugate with sign `cj` in
+// g unless null.  Returns false if a value is not finite.
+template <typename Rhs>
+__device__ __forceinline__ bool band_solve(const TcDev& d, const double* __restrict__ lu, int k, int pair, double* f, double* g,
+                                           double cj, Rhs rhs) {
+    const int N = d.Nr;
+    const size_t P2 = 2 * (size_t)d.npairs;
+    double y1 = 0.0, y2 = 0.0;                  // y_(j-1), y_(j-2)
+    rows_ahead<FwdRow>(
+        N - 2,
+        [&](int q, FwdRow& w) {
+            const int j = q + 1;
+            w.r = rhs(j);
+            w.m2 = TAB(lu, k, j, 0);
+            w.m1 = TAB(lu, k, j, 1);
+        },
+        [&](int q, const FwdRow& w) {
+            const double y = fma(-w.m1, y1, fma(-w.m2, y2, w.r));
+            f[(size_t)(q + 1) * P2] = y;
+            y2 = y1; y1 = y;
+        });
+    bool ok = true;
+    double x1 = 0.0, x2 = 0.0;                  // x_(i+1), x_(i+2)
+    rows_ahead<BackRow>(
+        N - 2,
+        [&](int q, BackRow& w) {
+            const int i = N - 2 - q;
+            w.y = f[(size_t)i * P2];
+            w.inv = TAB(lu, k, i, 2);
+            w.c = TAB(lu, k, i, 3);
+            w.e = TAB(lu, k, i, 4);
+        },
+        [&](int q, const BackRow& w) {
+            const int i = N - 2 - q;
+            const double x = w.inv * fma(-w.e, x2, fma(-w.c, x1, w.y));
+            ok = ok && dfinite(x);
+            f[(size_t)i * P2] = x;
+            if (g) g[(size_t)i * P2] = cj * x;
+            x2 = x1; x1 = x;
+        });
+    f[0] = 0.0;
+    f[(size_t)(N - 1) * P2] = 0.0;
+    if (g) { g[0] = 0.0; g[(size_t)(N - 1) * P2] = 0.0; }
+    return ok;
 }
 
-// Kernel variants: a register budget from launch bounds (threads per block,
-// resident blocks per SM), or an explicit register cap.
-template <int MODE, int MAXT, int MINB, bool NOH = false>
-__global__ void __launch_bounds__(MAXT, MINB) k_line(TcDev d, int k, int ja, int jw) {
-    line_body<MODE, NOH>(d, k, ja, jw, blockIdx.x * blockDim.x + threadIdx.x);
+// l1 . v on the rows i0 <= i < i1 of 1 .. Nr - 2 (one-sided on the first and the
+// last: Dv itself), into S: the right sides of the Dv solve.
+__device__ __forceinline__ void derivative_rows(const TcDev& d, const RowTables& t, const double* v, double* S, int i0, int i1) {
+    const int N = d.Nr;
+    const size_t P2 = 2 * (size_t)d.npairs, S2 = 2 * (size_t)d.Mzx * d.Nh;
+    i0 = i0 < 2 ? 2 : i0;
+    i1 = i1 > N - 2 ? N - 2 : i1;
+    if (i0 >= i1) return;
+    double x[5];
+    for (int s = 0; s < 4; ++s) x[s + 1] = v[(i0 - 2 + s) * P2];
+    auto row = [&](int j) {
+        double acc = 0.0;
+        for (int s = 0; s < 5; ++s) acc = fma(t.l1[j * 5 + s], x[s], acc);
+        S[(size_t)j * S2] = acc;
+    };
+    for (int i = i0; i < i1; ++i) {
+        for (int s = 0; s < 4; ++s) x[s] = x[s + 1];
+        x[4] = v[(i + 2) * P2];
+        row(i);
+        if (i == 2) row(1);
+        if (i == N - 3) row(N - 2);
+    }
 }
-template <int MODE, int NREG, bool NOH = false>
-__global__ void __maxnreg__(NREG) k_line_r(TcDev d, int k, int ja, int jw) {
-    line_body<MODE, NOH>(d, k, ja, jw, blockIdx.x * blockDim.x + threadIdx.x);
+// Dv in S: 0 on the walls; explicit one-sided rows 1 and Nr - 2 (there already);
+// compact rows d0 . Dv = l1 . v on rows 2 .. Nr - 3, solved with the reversed
+// factorisation dsol, whose elimination runs from the outer wall in.
+__device__ __forceinline__ void derivative_solve(const TcDev& d, const RowTables& t, double* S) {
+    const int N = d.Nr;
+    const size_t S2 = 2 * (size_t)d.Mzx * d.Nh;
+    const double D1 = S[S2], DN = S[(size_t)(N - 2) * S2];
+    double z1 = 0.0, z2 = 0.0;
+    rows_ahead<OneRow>(
+        N - 4, [&](int q, OneRow& w) { w.z = S[(size_t)(N - 3 - q) * S2]; },
+        [&](int q, const OneRow& w) {
+            const int j = N - 3 - q;
+            const double* w0 = t.d0 + j * 5;
+            double r = w.z;
+            if (j == N - 3) r = fma(-w0[3], DN, r);
+            if (j == N - 4) r = fma(-w0[4], DN, r);
+            if (j == 2) r = fma(-w0[1], D1, r);
+            if (j == 3) r = fma(-w0[0], D1, r);
+            const double* c = t.dsol + j * 5;
+            const double z = fma(-c[1], z1, fma(-c[0], z2, r));
+            S[(size_t)j * S2] = z;
+            z2 = z1; z1 = z;
+        });
+    double p1 = 0.0, p2 = 0.0;
+    rows_ahead<OneRow>(
+        N - 4, [&](int q, OneRow& w) { w.z = S[(size_t)(q + 2) * S2]; },
+        [&](int q, const OneRow& w) {
+            const double* c = t.dsol + (q + 2) * 5;
+            const double Dv = c[2] * fma(-c[4], p2, fma(-c[3], p1, w.z));
+            S[(size_t)(q + 2) * S2] = Dv;
+            p2 = p1; p1 = Dv;
+        });
+    S[0] = 0.0;
+    S[(size_t)(N - 1) * S2] = 0.0;
 }
-// Split variant for few pairs (a short line phase is bound by the latency
-// of one thread's radial recurrences): blocks of 64 threads, the first warp
-// advances v and the second eta of the same 32 pairs, then, after the block
-// barrier, the first warp rebuilds u and w.  The same arithmetic per field
-// as k_line.
-template <int MODE, bool NOH = false>
-__global__ void __launch_bounds__(64) k_line_s(TcDev d, int k, int ja, int jw) {
-    const int lane = threadIdx.x & 31;
-    const bool vrole = threadIdx.x < 32;
-    const int idx = blockIdx.x * 32 + lane;
+// u = (i alpha D_*v - (i m/r) eta)/k^2,   w = ((i m/r) D_*v + i alpha eta)/k^2 on the
+// rows i0 <= i < i1: the factor i takes each lane's value to the other component.
+__device__ __forceinline__ void velocity_rows(const TcDev& d, const RowTables& t, int pair, int comp, double m, double al,
+                                              long long partner, const double* S, int i0, int i1) {
+    const size_t P = d.npairs, P2 = 2 * P, S2 = 2 * (size_t)d.Mzx * d.Nh;
+    const size_t o = 2 * (size_t)pair + comp, x = 2 * (size_t)pair + 1 - comp;
+    const double *v = reinterpret_cast<const double*>(d.v) + o, *e = reinterpret_cast<const double*>(d.eta) + o;
+    double *u = reinterpret_cast<double*>(d.u), *w = reinterpret_cast<double*>(d.w);
+    for (int i = i0; i < i1; ++i) {
+        const double ri = t.rinv[i], c = d.tab_c[(size_t)i * P + pair];
+        const double Dsv = fma(ri, v[(size_t)i * P2], S[(size_t)i * S2]), E = e[(size_t)i * P2];
+        const double ca = c * al, cm = c * m * ri;
+        const double su = fma(ca, Dsv, -cm * E), sw = fma(cm, Dsv, ca * E);
+        u[x + (size_t)i * P2] = comp ? -su : su;
+        w[x + (size_t)i * P2] = comp ? -sw : sw;
+        if (partner >= 0) {
+            u[2 * (size_t)partner + 1 - comp + (size_t)i * P2] = -su;
+            w[2 * (size_t)partner + 1 - comp + (size_t)i * P2] = -sw;
+        }
+    }
+}
+
+template <bool NOH>
+__device__ __forceinline__ void solve_body(const TcDev& d, int k, int ja, int jw, int block) {
+    const int warp = threadIdx.x >> 5, comp = threadIdx.x & 1;
     int pair = 0;
     double m = 0.0, al = 0.0;
     long long partner = -1;
-    bool act;
-    if (vrole) act = line_sweeps<MODE, 1, NOH>(d, k, ja, jw, idx, pair, m, al, partner);
-    else act = line_sweeps<MODE, 2, NOH>(d, k, ja, jw, idx, pair, m, al, partner);
-    __syncthreads();
-    if (vrole && act) reconstruct_pair(d, pair, m, al, partner);
-}
-
-// The implicit part of the next RK memory (rk_memory_row) for the pairs of
-// the columns ja .. ja + jw - 1, after a line kernel of substep k launched
-// with NOH: one thread per pair walks its radial line downwards like the
-// back substitution, reading x^(k+1) (v, eta) instead of computing it.  It
-// needs only the results of that line kernel, so it can run beside the next
-// substep's plane phase.
-// Grid-stride over the pairs: launched beside the theta rows it runs in few
-// blocks (four per SM), so that it takes mostly what the rows leave free.
-__global__ void __launch_bounds__(128) k_rk_memory(TcDev d, int k, int ja, int jw) {
+    const bool act = line_pair(d, ja, jw, block * 16 + ((threadIdx.x & 31) >> 1), pair, m, al, partner);
     const int N = d.Nr;
-    const size_t P = d.npairs;
-    const int kn = (k + 1) % 3;
-    const double hdt = (d.rk_beta[k] + d.rk_alpha[kn]) * d.dt;
-    const double hdtnu = hdt * d.nu;
-    const int n = d.Nz * jw;
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += gridDim.x * blockDim.x) {
-        const int pair = (idx / jw) * d.Nh + ja + idx % jw;
-        double m, al;
-        long long partner;
-        if (!pair_info(d, pair, m, al, partner)) continue;
-        double2 xw[5], ew[5];
-        double k2w[5];
-        for (int s = 0; s < 5; ++s) { xw[s] = cz(); ew[s] = cz(); k2w[s] = 0.0; }
-        k2w[0] = k2_at(m, al, d.rinv[N - 1]);
-        for (int i = N - 2; i >= 0; --i) {
-            for (int s = 4; s > 0; --s) { xw[s] = xw[s - 1]; ew[s] = ew[s - 1]; k2w[s] = k2w[s - 1]; }
-            k2w[0] = k2_at(m, al, d.rinv[i]);
-            if (i >= 1) {
-                xw[0] = d.v[(size_t)i * P + pair];
-                ew[0] = d.eta[(size_t)i * P + pair];
-            } else {
-                xw[0] = cz(); ew[0] = cz();
-            }
-            if (i == N - 5) rk_memory_row(d, pair, N - 2, xw, ew, k2w, hdt, hdtnu, false, true);
-            const int jr = i + 2;
-            if (i <= N - 5 && jr >= 2) rk_memory_row(d, pair, jr, xw, ew, k2w, hdt, hdtnu, true, true);
-            if (i == 0) rk_memory_row(d, pair, 1, xw, ew, k2w, hdt, hdtnu, false, true);
+    const RowTables t{d.d0, d.l1, d.dsol, d.rinv};
+    const size_t o = 2 * (size_t)pair + comp, P2 = 2 * (size_t)d.npairs, S2 = 2 * (size_t)d.Mzx * d.Nh;
+    double* S = reinterpret_cast<double*>(rhs_scratch(d, pair)) + comp;
+    double* const v = reinterpret_cast<double*>(d.v) + o;
+    if (act) {
+        const double cj = comp ? -1.0 : 1.0;
+        bool ok;
+        if (warp == 0) {
+            const double fv = TAB(d.tab_luv, k, 0, 0), gv = TAB(d.tab_luv, k, N - 1, 0);
+            ok = band_solve(d, d.tab_luv, k, pair, v, partner >= 0 ? reinterpret_cast<double*>(d.v) + 2 * partner + comp : nullptr, cj,
+                            [&](int j) { return j == 1 ? -fv * S[2 * S2] : j == N - 2 ? -gv * S[(size_t)(N - 3) * S2] : S[(size_t)j * S2]; });
+        } else {
+            double* const e = reinterpret_cast<double*>(d.eta) + o;
+            const double fe = TAB(d.tab_lue, k, 0, 0), ge = TAB(d.tab_lue, k, N - 1, 0);
+            // the folded right sides, before y overwrites the rows they use
+            const double e1 = fma(-fe, e[2 * P2], e[P2]), eN = fma(-ge, e[(size_t)(N - 3) * P2], e[(size_t)(N - 2) * P2]);
+            ok = band_solve(d, d.tab_lue, k, pair, e, partner >= 0 ? reinterpret_cast<double*>(d.eta) + 2 * partner + comp : nullptr, cj,
+                            [&](int j) { return j == 1 ? e1 : j == N - 2 ? eN : e[(size_t)j * P2]; });
         }
+        if (!ok) atomicOr(d.flag, 1);
+    }
+    const int i0 = warp * N / 2, i1 = (warp + 1) * N / 2;      // the warp's share of the radial rows
+    __syncthreads();
+    if (act) derivative_rows(d, t, v, S, i0, i1);
+    __syncthreads();
+    if (act && warp == 0) derivative_solve(d, t, S);
+    __syncthreads();
+    if (act) {
+        if (!NOH) rk_memory_rows(d, k, pair, comp, i0, i1);
+        velocity_rows(d, t, pair, comp, m, al, partner, S, i0, i1);
     }
 }
 
-// Many cases in one launch: blocks of 128 threads, bmap[block] = (case,
-// block within the case), the case's descriptor from ds.
-template <int MODE>
-__global__ void __launch_bounds__(128, 4) k_line_b(const TcDev* __restrict__ ds, const int2* __restrict__ bmap, int k) {
-    const int2 m = bmap[blockIdx.x];
-    const TcDev& d = ds[m.x];
-    line_body<MODE>(d, k, 0, d.Nh, m.y * blockDim.x + threadIdx.x);
+// The same for few pairs: eight warps, of which the recurrences still have one each, so
+// that what counts is the time of one row of them.  The factors come through a ring in
+// shared memory (cp.async, 16 rows deep: the latency of a load is several rows), and
+// what one sweep leaves for the next (y, x, the right sides and z of the Dv solve)
+// stays in shared memory.  Same operations, same bits.  Line phase of
+// 129x128x128 623 -> 536 us, mixed form 437 -> 350.
+constexpr int SOLVE_WARPS = 8, RING_ROWS = 16;
+struct DvRow { double z, a, b, c; };
+struct RkRow { double tv[5], te[5], Hv, He, e; };
+struct VelRow { double c, e; };
+// n rows of three words each per lane, p[w] + row stride[w], four rows at a time.  A
+// lone warp issues an instruction every few cycles, so the sources are pointers that
+// advance, not indexed tables.
+struct Ring3 { const double* p[3]; long long stride[3]; };
+template <typename Step> __device__ __forceinline__ void ring_rows(double* ring, int n, Ring3 s, Step step) {
+    constexpr int B = 4, NB = RING_ROWS / B;
+    double* const mine = ring + (threadIdx.x & 31);
+    int left = n;
+    auto issue = [&](int slot) {
+        double* o = mine + slot * (B * 96);
+#pragma unroll
+        for (int q = 0; q < B; ++q) {
+            if (q < left)
+#pragma unroll
+                for (int w = 0; w < 3; ++w) {
+                    copy_async<8>(o + (q * 3 + w) * 32, s.p[w]);
+                    s.p[w] += s.stride[w];
+                }
+        }
+        left -= B;
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int b = 0; b < NB - 1; ++b) issue(b);
+    for (int b = 0; b < n; b += B) {
+        issue((b / B + NB - 1) % NB);
+        asm volatile("cp.async.wait_group %0;" ::"n"(NB - 1) : "memory");
+        const double* o = mine + (b / B % NB) * (B * 96);
+        double w[B][3];
+#pragma unroll
+        for (int q = 0; q < B; ++q)
+#pragma unroll
+            for (int t = 0; t < 3; ++t) w[q][t] = o[(q * 3 + t) * 32];
+#pragma unroll
+        for (int q = 0; q < B; ++q)
+            if (b + q < n) step(b + q, w[q]);
+    }
+}
+// band_solve on the ring: right sides at r + j S2 but r1 and rN for rows 1 and Nr - 2; y
+// and then x in Y, x in f as well
+__device__ __forceinline__ bool band_solve_shared(const TcDev& d, const double* __restrict__ lu, int k, int pair, double* ring, double* Y,
+                                                  double* f, double* g, double cj, const double* r, size_t S2, double r1, double rN) {
+    const int N = d.Nr;
+    const long long P = d.npairs, P2 = 2 * P;
+    double y1 = 0.0, y2 = 0.0;
+    double* Yq = Y + 32;
+    const double* l = &TAB(lu, k, 1, 0);
+    ring_rows(ring, N - 2, Ring3{{r + S2, l, l + P}, {(long long)S2, 5 * P, 5 * P}}, [&](int q, const double* w) {
+        const double b = q == 0 ? r1 : q == N - 3 ? rN : w[0];
+        const double y = fma(-w[2], y1, fma(-w[1], y2, b));
+        *Yq = y;
+        Yq += 32;
+        y2 = y1; y1 = y;
+    });
+    unsigned top = 0;                           // largest exponent field
+    double x1 = 0.0, x2 = 0.0;
+    f += (N - 2) * P2;
+    if (g) g += (N - 2) * P2;
+    l = &TAB(lu, k, N - 2, 2);
+    ring_rows(ring, N - 2, Ring3{{l, l + P, l + 2 * P}, {-5 * P, -5 * P, -5 * P}}, [&](int q, const double* w) {
+        Yq -= 32;
+        const double x = w[0] * fma(-w[2], x2, fma(-w[1], x1, *Yq));
+        const unsigned ex = (unsigned)__double2hiint(x) & 0x7ff00000u;
+        top = ex > top ? ex : top;
+        *Yq = x;
+        *f = x;
+        f -= P2;
+        if (g) { *g = cj * x; g -= P2; }
+        x2 = x1; x1 = x;
+    });
+    Y[0] = Y[(N - 1) * 32] = 0.0;
+    f[0] = f[(N - 1) * P2] = 0.0;
+    if (g) g[0] = g[(N - 1) * P2] = 0.0;
+    return top != 0x7ff00000u;
+}
+template <bool NOH>
+__device__ __forceinline__ void solve_shared_body(const TcDev& d, int k, int ja, int jw, int block) {
+    extern __shared__ double sm[];
+    const int N = d.Nr, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, comp = threadIdx.x & 1;
+    double *const d0 = sm, *const l1 = d0 + 5 * N, *const dsol = l1 + 5 * N, *const rinv = dsol + 5 * N;
+    double *const V = rinv + N + lane, *const D = V + 32 * N;               // D: y of eta before
+    double* const ring = rinv + N + 64 * N + warp * RING_ROWS * 96;         // of warps 0 and 1
+    for (int i = threadIdx.x; i < 5 * N; i += 32 * SOLVE_WARPS) { d0[i] = d.d0[i]; l1[i] = d.l1[i]; dsol[i] = d.dsol[i]; }
+    for (int i = threadIdx.x; i < N; i += 32 * SOLVE_WARPS) rinv[i] = d.rinv[i];
+    int pair = 0;
+    double m = 0.0, al = 0.0;
+    long long partner = -1;
+    const bool act = line_pair(d, ja, jw, block * 16 + (lane >> 1), pair, m, al, partner);
+    const size_t P = d.npairs, P2 = 2 * P, S2 = 2 * (size_t)d.Mzx * d.Nh, o = 2 * (size_t)pair + comp;
+    const double* S = reinterpret_cast<const double*>(rhs_scratch(d, pair)) + comp;
+    double *const v = reinterpret_cast<double*>(d.v) + o, *const e = reinterpret_cast<double*>(d.eta) + o;
+    if (act && warp < 2) {
+        const double cj = comp ? -1.0 : 1.0;
+        bool ok;
+        if (warp == 0) {
+            const double r1 = -TAB(d.tab_luv, k, 0, 0) * S[2 * S2], rN = -TAB(d.tab_luv, k, N - 1, 0) * S[(size_t)(N - 3) * S2];
+            ok = band_solve_shared(d, d.tab_luv, k, pair, ring, V, v, partner >= 0 ? reinterpret_cast<double*>(d.v) + 2 * partner + comp : nullptr,
+                                   cj, S, S2, r1, rN);
+        } else {
+            const double fe = TAB(d.tab_lue, k, 0, 0), ge = TAB(d.tab_lue, k, N - 1, 0);
+            const double e1 = fma(-fe, e[2 * P2], e[P2]), eN = fma(-ge, e[(size_t)(N - 3) * P2], e[(size_t)(N - 2) * P2]);
+            ok = band_solve_shared(d, d.tab_lue, k, pair, ring, D, e, partner >= 0 ? reinterpret_cast<double*>(d.eta) + 2 * partner + comp : nullptr,
+                                   cj, e, P2, e1, eN);
+        }
+        if (!ok) atomicOr(d.flag, 1);
+    }
+    __syncthreads();
+    // l1 . v
+    for (int j = 1 + warp; j < N - 1; j += SOLVE_WARPS) {
+        const int st = j == 1 ? 0 : j == N - 2 ? N - 5 : j - 2;
+        double acc = 0.0;
+        for (int s = 0; s < 5; ++s) acc = fma(l1[j * 5 + s], V[(st + s) * 32], acc);
+        D[j * 32] = acc;
+    }
+    __syncthreads();
+    // the Dv recurrences, the RK memory beside them
+    if (warp == 0) {
+        const double D1 = D[32], DN = D[(N - 2) * 32];
+        double *Dq = D + (N - 3) * 32, *q = dsol + (N - 3) * 5;
+        D[(N - 3) * 32] = fma(-d0[(N - 3) * 5 + 3], DN, D[(N - 3) * 32]);
+        D[(N - 4) * 32] = fma(-d0[(N - 4) * 5 + 4], DN, D[(N - 4) * 32]);
+        D[64] = fma(-d0[11], D1, D[64]);
+        D[96] = fma(-d0[15], D1, D[96]);
+        double z1 = 0.0, z2 = 0.0;
+        rows_ahead<DvRow>(
+            N - 4,
+            [&](int, DvRow& w) {
+                w.z = *Dq; w.a = q[0]; w.b = q[1];
+                Dq -= 32; q -= 5;
+            },
+            [&](int r, const DvRow& w) {
+                const double z = fma(-w.b, z1, fma(-w.a, z2, w.z));
+                D[(N - 3 - r) * 32] = z;
+                z2 = z1; z1 = z;
+            });
+        double p1 = 0.0, p2 = 0.0;
+        Dq = D + 64;
+        q = dsol + 10;
+        rows_ahead<DvRow>(
+            N - 4,
+            [&](int, DvRow& w) {
+                w.z = *Dq; w.a = q[2]; w.b = q[3]; w.c = q[4];
+                Dq += 32; q += 5;
+            },
+            [&](int r, const DvRow& w) {
+                const double x = w.a * fma(-w.c, p2, fma(-w.b, p1, w.z));
+                D[(2 + r) * 32] = x;
+                p2 = p1; p1 = x;
+            });
+        D[0] = D[(N - 1) * 32] = 0.0;
+    } else if (act && !NOH) {
+        const int n = SOLVE_WARPS - 1, i0 = 2 + (warp - 1) * (N - 4) / n, i1 = 2 + warp * (N - 4) / n;
+        const double hdt = (d.rk_beta[k] + d.rk_alpha[(k + 1) % 3]) * d.dt, hdtnu = hdt * d.nu;
+        double *Hv = reinterpret_cast<double*>(d.Hv) + o, *He = reinterpret_cast<double*>(d.He) + o;
+        double xe[5];
+        if (i0 < i1)
+            for (int s = 0; s < 4; ++s) xe[s + 1] = e[(i0 - 2 + s) * P2];
+        rows_ahead<RkRow, 1>(
+            i1 - i0,
+            [&](int q, RkRow& w) {
+                const int i = i0 + q;
+#pragma unroll
+                for (int s = 0; s < 5; ++s) { w.tv[s] = TAB(d.tab_lv, 0, i, s); w.te[s] = TAB(d.tab_le, 0, i, s); }
+                w.Hv = Hv[(size_t)i * P2];
+                w.He = He[(size_t)i * P2];
+                w.e = e[(size_t)(i + 2) * P2];
+            },
+            [&](int q, const RkRow& w) {
+                const int i = i0 + q;
+                for (int s = 0; s < 4; ++s) xe[s] = xe[s + 1];
+                xe[4] = w.e;
+                double av = 0.0, ae = 0.0;
+#pragma unroll
+                for (int s = 0; s < 5; ++s) { av = fma(w.tv[s], V[(i - 2 + s) * 32], av); ae = fma(w.te[s], xe[s], ae); }
+                Hv[(size_t)i * P2] = fma(hdt, av, w.Hv);
+                He[(size_t)i * P2] = fma(hdtnu, ae, w.He);
+                if (i == 2) rk_memory_row(d, d.tab_le, He, pair, 1, xe, hdtnu);
+                if (i == N - 3) rk_memory_row(d, d.tab_le, He, pair, N - 2, xe, hdtnu);
+            });
+    }
+    __syncthreads();
+    if (!act) return;
+    // u and w: as in velocity_rows
+    const size_t x = 2 * (size_t)pair + 1 - comp;
+    double *u = reinterpret_cast<double*>(d.u), *w = reinterpret_cast<double*>(d.w);
+    const int n = (N - warp + SOLVE_WARPS - 1) / SOLVE_WARPS;
+    rows_ahead<VelRow, 2>(
+        n,
+        [&](int q, VelRow& r) {
+            const size_t i = warp + q * SOLVE_WARPS;
+            r.c = d.tab_c[i * P + pair];
+            r.e = e[i * P2];
+        },
+        [&](int q, const VelRow& r) {
+            const size_t i = warp + q * SOLVE_WARPS;
+            const double ri = rinv[i];
+            const double Dsv = fma(ri, V[i * 32], D[i * 32]);
+            const double ca = r.c * al, cm = r.c * m * ri;
+            const double su = fma(ca, Dsv, -cm * r.e), sw = fma(cm, Dsv, ca * r.e);
+            u[x + i * P2] = comp ? -su : su;
+            w[x + i * P2] = comp ? -sw : sw;
+            if (partner >= 0) {
+                u[2 * (size_t)partner + 1 - comp + i * P2] = -su;
+                w[2 * (size_t)partner + 1 - comp + i * P2] = -sw;
+            }
+        });
+}
+static size_t solve_smem(int Nr) { return (80 * (size_t)Nr + 2 * RING_ROWS * 96) * sizeof(double); }
+// Which of the two: up to WIDE_GROUPS blocks of 16 pairs.  Line phase with
+// two and with eight warps: 512 blocks (129x128x128) 623 and 536 us, 2720 (129x512x170)
+// 2.39 and 2.47 ms, 8192 (257x512x512) 13.4 and 19.2 ms.
+constexpr long long WIDE_GROUPS = 8 * 152;
+static bool solve_wide(long long groups, int Nr) { return groups < WIDE_GROUPS && solve_smem(Nr) <= 200 * 1024; }
+
+// The implicit part of the next RK memory (rk_memory_row) for the pairs of
+// the columns ja .. ja + jw - 1, after a k_solve of substep k launched with NOH:
+// one thread per pair and component walks its radial line.  It needs only the
+// results of that kernel, so it can run beside the next substep's plane phase.
+// Grid-stride over the pairs: launched beside the theta rows it runs in few
+// blocks (four per SM), so that it takes mostly what the rows leave free.
+__global__ void __launch_bounds__(128) k_rk_memory(TcDev d, int k, int ja, int jw) {
+    const int n = 2 * d.Nz * jw;
+    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += gridDim.x * blockDim.x) {
+        int pair;
+        double m, al;
+        long long partner;
+        if (line_pair(d, ja, jw, idx >> 1, pair, m, al, partner)) rk_memory_rows(d, k, pair, idx & 1, 0, d.Nr);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -838,24 +1195,51 @@ __global__ void __launch_bounds__(128) k_init(TcDev d) {
 // Mean flow (m = alpha = 0), zero mean pressure gradient (Sec. 4):
 //   dW/dt = nu D D_* W - D(vw) - 2 vw/r,   dU/dt = nu (D D_* U + U/r^2) - D(uv) - uv/r,
 // rows 1..Nr-2 with Dirichlet values W(R_i) = 1, W(R_o) = Re_o/Re_i, U = 0.
-// One block: rows are assembled in parallel into shared memory, then two
-// threads run the banded eliminations (U and W) serially.
+// One block: the right sides in parallel, then one thread each for U and W runs
+// the banded solve with the factors of mean_lu (the system is the same in every
+// step), from shared memory: the recurrences are the latency of a few thousand
+// dependent operations, so nothing else is left in them.
+__device__ __forceinline__ void mean_L(const TcDev& d, int j, int s, double& lu, double& lw) {
+    const double w0 = d.d0[j * 5 + s], w2 = d.l2[j * 5 + s], ri = d.rinv[d.start[j] + s];
+    lu = d.nu * (w2 + w0 * ri * ri);
+    lw = d.nu * w2;
+}
+// H_1 = (M + alpha_1 dt L) x, and u(0,0) = U, w(0,0) = W
+__global__ void __launch_bounds__(256) k_mean_init(TcDev d) {
+    const int N = d.Nr;
+    const double adt = d.rk_alpha[0] * d.dt;
+    for (int j = threadIdx.x; j < N; j += blockDim.x) {
+        double hu = 0.0, hw = 0.0;
+        if (j >= 1 && j <= N - 2) {
+            const int st = d.start[j];
+            for (int s = 0; s < 5; ++s) {
+                double lu, lw;
+                mean_L(d, j, s, lu, lw);
+                hu += (d.d0[j * 5 + s] + adt * lu) * d.U[st + s];
+                hw += (d.d0[j * 5 + s] + adt * lw) * d.W[st + s];
+            }
+        }
+        d.HU[j] = hu;
+        d.HW[j] = hw;
+        d.u[(size_t)j * d.npairs] = make_double2(d.U[j], 0.0);
+        d.w[(size_t)j * d.npairs] = make_double2(d.W[j], 0.0);
+    }
+}
 template <typename PT>
-__device__ __forceinline__ void mean_body(const TcDev& d, int k, int init) {
+__device__ __forceinline__ void mean_body(const TcDev& d, int k) {
     extern __shared__ double sm[];
     const int N = d.Nr;
-    double* A = sm;                    // [2][N][5] system rows
-    double* Lb = A + 2 * N * 5;        // [2][N][5] implicit rows
-    double* rhs = Lb + 2 * N * 5;      // [2][N]
+    double* lu = sm;                   // [2][N][5] factors of this substep
+    double* rhs = lu + 2 * N * 5;      // [2][N]
     double* x = rhs + 2 * N;           // [2][N]
-    double* Ex = x + 2 * N;            // [2][N] explicit rows
     const PT* prod = reinterpret_cast<const PT*>(d.prod);
     const size_t PS = (size_t)N * d.npairs;
     const int kn = (k + 1) % 3;
     const double bdt = d.rk_beta[k] * d.dt;
-    for (int j = threadIdx.x; j < N; j += blockDim.x) {
-        x[j] = d.U[j];
-        x[N + j] = d.W[j];
+    const double gdt = d.rk_gamma[k] * d.dt, zdt = d.rk_zeta[kn] * d.dt;
+    for (int i = threadIdx.x; i < 10 * N; i += blockDim.x) {
+        const int p = i / (5 * N);
+        lu[i] = d.mean_lu[(size_t)(p * 3 + k) * N * 5 + (i - p * 5 * N)];
     }
     for (int j = threadIdx.x; j < N; j += blockDim.x) {
         if (j < 1 || j > N - 2) continue;
@@ -863,125 +1247,52 @@ __device__ __forceinline__ void mean_body(const TcDev& d, int k, int init) {
         double eu = 0.0, ew = 0.0;
         for (int s = 0; s < 5; ++s) {
             const int i = st + s;
-            const double w0 = d.d0[j * 5 + s], w1 = d.l1[j * 5 + s], w2 = d.l2[j * 5 + s];
-            const double ri = d.rinv[i];
-            Lb[(0 * N + j) * 5 + s] = d.nu * (w2 + w0 * ri * ri);   // U
-            Lb[(1 * N + j) * 5 + s] = d.nu * w2;                    // W
-            if (!init) {
-                const double uv = ld_prod(prod, (size_t)i * d.npairs + PS).x;
-                const double vw = ld_prod(prod, (size_t)i * d.npairs + 3 * PS).x;
-                eu += -w1 * uv - w0 * uv * ri;
-                ew += -w1 * vw - 2.0 * w0 * vw * ri;
-            }
+            const double w0 = d.d0[j * 5 + s], w1 = d.l1[j * 5 + s], ri = d.rinv[i];
+            const double uv = ld_prod(prod, (size_t)i * d.npairs + PS).x;
+            const double vw = ld_prod(prod, (size_t)i * d.npairs + 3 * PS).x;
+            eu += -w1 * uv - w0 * uv * ri;
+            ew += -w1 * vw - 2.0 * w0 * vw * ri;
         }
-        Ex[j] = eu;
-        Ex[N + j] = ew;
+        double ru = d.HU[j] + gdt * eu, rw = d.HW[j] + gdt * ew;
+        d.HU[j] = ru + zdt * eu;
+        d.HW[j] = rw + zdt * ew;
+        // the Dirichlet values W(r_0) = 1, W(r_(N-1)) = W_outer to the right side (U: 0)
+        double a, b;
+        if (st == 0) { mean_L(d, j, 0, a, b); rw -= d.d0[j * 5] - bdt * b; }
+        if (st + 4 == N - 1) { mean_L(d, j, 4, a, b); rw -= (d.d0[j * 5 + 4] - bdt * b) * d.W_outer; }
+        rhs[j] = ru;
+        rhs[N + j] = rw;
     }
     __syncthreads();
-    if (init) {
-        // H_1 = (M + alpha_1 dt L) x, and u(0,0) = U, w(0,0) = W
-        const double adt = d.rk_alpha[0] * d.dt;
-        for (int j = threadIdx.x; j < N; j += blockDim.x) {
-            double hu = 0.0, hw = 0.0;
-            if (j >= 1 && j <= N - 2) {
-                const int st = d.start[j];
-                for (int s = 0; s < 5; ++s) {
-                    hu += (d.d0[j * 5 + s] + adt * Lb[j * 5 + s]) * x[st + s];
-                    hw += (d.d0[j * 5 + s] + adt * Lb[(N + j) * 5 + s]) * x[N + st + s];
-                }
-            }
-            d.HU[j] = hu;
-            d.HW[j] = hw;
-            d.u[(size_t)j * d.npairs] = make_double2(x[j], 0.0);
-            d.w[(size_t)j * d.npairs] = make_double2(x[N + j], 0.0);
-        }
-        return;
-    }
-    // right sides and system rows
-    const double gdt = d.rk_gamma[k] * d.dt, zdt = d.rk_zeta[kn] * d.dt;
-    for (int j = threadIdx.x; j < N; j += blockDim.x) {
-        for (int p = 0; p < 2; ++p) {
-            double* H = p == 0 ? d.HU : d.HW;
-            if (j >= 1 && j <= N - 2) {
-                const double rr = H[j] + gdt * Ex[p * N + j];
-                rhs[p * N + j] = rr;
-                H[j] = rr + zdt * Ex[p * N + j];
-                for (int s = 0; s < 5; ++s)
-                    A[(p * N + j) * 5 + s] = d.d0[j * 5 + s] - bdt * Lb[(p * N + j) * 5 + s];
-            }
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x < 2) {
-        const int p = threadIdx.x;
-        const double b0 = p == 0 ? 0.0 : 1.0;                 // value at r_0
-        const double bN = p == 0 ? 0.0 : d.W_outer;           // value at r_{N-1}
-        double* Ap = A + p * N * 5;
+    if (threadIdx.x % 32 == 0 && threadIdx.x / 32 < 2) {
+        const int p = threadIdx.x / 32;
+        const double* q = lu + p * N * 5;
         double* rp = rhs + p * N;
         double* xp = x + p * N;
-        // move the Dirichlet columns to the right side
-        for (int j = 1; j <= N - 2; ++j) {
-            const int st = d.start[j];
-            if (st == 0) { rp[j] -= Ap[j * 5 + 0] * b0; Ap[j * 5 + 0] = 0.0; }
-            if (st + 4 == N - 1) { rp[j] -= Ap[j * 5 + 4] * bN; Ap[j * 5 + 4] = 0.0; }
-        }
-        // reduced rows on unknowns 1..N-2: (a, b, d, c, e) about the diagonal
-        auto reduced = [&](int j, double* R) {
-            const int off = d.start[j] - (j - 2);   // 0 for centred rows
-            for (int t = 0; t < 5; ++t) R[t] = 0.0;
-            for (int s = 0; s < 5; ++s) {
-                const int t = s + off;
-                if (t >= 0 && t < 5) R[t] = Ap[j * 5 + s];
-            }
-        };
-        // row 1 reaches column 4 (t = 5) and row N-2 column N-5 (t = -1):
-        // fold them with rows 2 and N-3
-        double R1[5], R2[5], R3[5], RN[5];
-        reduced(2, R2);
-        reduced(N - 3, R3);
-        {
-            const double f = Ap[1 * 5 + 4] / R2[4];
-            for (int t = 0; t < 5; ++t) R1[t] = 0.0;
-            R1[2] = Ap[1 * 5 + 1] - f * R2[1];
-            R1[3] = Ap[1 * 5 + 2] - f * R2[2];
-            R1[4] = Ap[1 * 5 + 3] - f * R2[3];
-            rp[1] -= f * rp[2];
-            const double g = Ap[(N - 2) * 5 + 0] / R3[0];
-            for (int t = 0; t < 5; ++t) RN[t] = 0.0;
-            RN[0] = Ap[(N - 2) * 5 + 1] - g * R3[1];
-            RN[1] = Ap[(N - 2) * 5 + 2] - g * R3[2];
-            RN[2] = Ap[(N - 2) * 5 + 3] - g * R3[3];
-            rp[N - 2] -= g * rp[N - 3];
-        }
-        // forward elimination (multipliers in place of the row)
-        double p2d = 1, p2c = 0, p2e = 0, p1d = 1, p1c = 0, p1e = 0;
+        rp[1] -= q[0] * rp[2];                          // fold the one-sided rows
+        rp[N - 2] -= q[(N - 1) * 5] * rp[N - 3];
         double y1 = 0, y2 = 0;
-        double* U3 = Lb + p * N * 5;                     // reuse: (1/d, c, e)
-        for (int i = 1; i <= N - 2; ++i) {
-            double R[5];
-            if (i == 1) for (int t = 0; t < 5; ++t) R[t] = R1[t];
-            else if (i == N - 2) for (int t = 0; t < 5; ++t) R[t] = RN[t];
-            else reduced(i, R);
-            const double m2 = (i >= 3) ? R[0] / p2d : 0.0;
-            double b = R[1] - m2 * p2c, dd = R[2] - m2 * p2e;
-            const double m1 = (i >= 2) ? b / p1d : 0.0;
-            dd -= m1 * p1c;
-            const double cc = R[3] - m1 * p1e;
-            const double y = rp[i] - m2 * y2 - m1 * y1;
-            U3[i * 5 + 0] = 1.0 / dd; U3[i * 5 + 1] = cc; U3[i * 5 + 2] = R[4];
-            rp[i] = y;
-            y2 = y1; y1 = y;
-            p2d = p1d; p2c = p1c; p2e = p1e;
-            p1d = dd; p1c = cc; p1e = R[4];
-        }
+        rows_ahead<MeanRow>(
+            N - 2, [&](int r, MeanRow& w) { w.y = rp[r + 1]; w.a = q[(r + 1) * 5]; w.b = q[(r + 1) * 5 + 1]; },
+            [&](int r, const MeanRow& w) {
+                const double y = fma(-w.b, y1, fma(-w.a, y2, w.y));
+                xp[r + 1] = y;
+                y2 = y1; y1 = y;
+            });
         double x1 = 0, x2 = 0;
-        for (int i = N - 2; i >= 1; --i) {
-            const double xi = (rp[i] - U3[i * 5 + 1] * x1 - U3[i * 5 + 2] * x2) * U3[i * 5 + 0];
-            xp[i] = xi;
-            x2 = x1; x1 = xi;
-        }
-        xp[0] = b0;
-        xp[N - 1] = bN;
+        rows_ahead<MeanRow>(
+            N - 2,
+            [&](int r, MeanRow& w) {
+                const int i = N - 2 - r;
+                w.y = xp[i]; w.a = q[i * 5 + 4]; w.b = q[i * 5 + 3]; w.inv = q[i * 5 + 2];
+            },
+            [&](int r, const MeanRow& w) {
+                const double x = w.inv * fma(-w.a, x2, fma(-w.b, x1, w.y));
+                xp[N - 2 - r] = x;
+                x2 = x1; x1 = x;
+            });
+        xp[0] = p == 0 ? 0.0 : 1.0;
+        xp[N - 1] = p == 0 ? 0.0 : d.W_outer;
     }
     __syncthreads();
     // H_(k+1) += (beta_k + alpha_(k+1)) dt L x, write the profiles
@@ -989,15 +1300,15 @@ __device__ __forceinline__ void mean_body(const TcDev& d, int k, int init) {
     for (int j = threadIdx.x; j < N; j += blockDim.x) {
         if (j >= 1 && j <= N - 2) {
             const int st = d.start[j];
-            double lu = 0.0, lw = 0.0;
+            double su = 0.0, sw = 0.0;
             for (int s = 0; s < 5; ++s) {
-                const int i = st + s;
-                const double w0 = d.d0[j * 5 + s], w2 = d.l2[j * 5 + s], ri = d.rinv[i];
-                lu += d.nu * (w2 + w0 * ri * ri) * x[i];
-                lw += d.nu * w2 * x[N + i];
+                double a, b;
+                mean_L(d, j, s, a, b);
+                su += a * x[st + s];
+                sw += b * x[N + st + s];
             }
-            d.HU[j] += hdt * lu;
-            d.HW[j] += hdt * lw;
+            d.HU[j] += hdt * su;
+            d.HW[j] += hdt * sw;
         }
         d.U[j] = x[j];
         d.W[j] = x[N + j];
@@ -1006,10 +1317,168 @@ __device__ __forceinline__ void mean_body(const TcDev& d, int k, int init) {
     }
 }
 template <typename PT>
-__global__ void __launch_bounds__(256) k_mean(TcDev d, int k, int init) { mean_body<PT>(d, k, init); }
-// one block per case of a shape class
-template <typename PT>
-__global__ void __launch_bounds__(256) k_mean_b(const TcDev* __restrict__ ds, int k) { mean_body<PT>(ds[blockIdx.x], k, 0); }
+__global__ void __launch_bounds__(256) k_mean(TcDev d, int k) { mean_body<PT>(d, k); }
+__device__ __forceinline__ void mean_any(const TcDev& d, int k) {
+    if (d.prec == 1) mean_body<float2>(d, k);
+    else if (d.prec == 2) mean_body<dcomplex>(d, k);
+    else mean_body<double2>(d, k);
+}
+
+// The solves of 16 pairs a block; with `mean`, the last block advances the mean flow.
+template <bool NOH>
+__global__ void __launch_bounds__(64, 12) k_solve(const __grid_constant__ TcDev d, int k, int ja, int jw) {
+    solve_body<NOH>(d, k, ja, jw, blockIdx.x);
+}
+template <bool NOH>
+__global__ void __launch_bounds__(32 * SOLVE_WARPS, 2) k_solve_shared(const __grid_constant__ TcDev d, int k, int ja, int jw, bool mean) {
+    if (mean && blockIdx.x == gridDim.x - 1) mean_any(d, k);
+    else solve_shared_body<NOH>(d, k, ja, jw, blockIdx.x);
+}
+// Many cases of one form in one launch: bmap[block] = (case, 16 pairs of the case;
+// -1: the case's mean flow)
+__global__ void __launch_bounds__(64, 12) k_solve_b(const TcDev* __restrict__ ds, const int2* __restrict__ bmap, int k) {
+    const int2 m = bmap[blockIdx.x];
+    solve_body<false>(ds[m.x], k, 0, ds[m.x].Nh, m.y);
+}
+__global__ void __launch_bounds__(32 * SOLVE_WARPS, 2)
+k_solve_shared_b(const TcDev* __restrict__ ds, const int2* __restrict__ bmap, int k) {
+    const int2 m = bmap[blockIdx.x];
+    const TcDev& d = ds[m.x];
+    if (m.y < 0) mean_any(d, k);
+    else solve_shared_body<false>(d, k, 0, d.Nh, m.y);
+}
+
+// The explicit rows, four warps a block: warp w of the launch takes chunk w % nch
+// (Lc rows each) of the 32 pairs w / nch, so that the warps of a block mostly share
+// the points at their chunks' ends.  With `mean`, the last block advances the mean
+// flow, which needs the products only.
+template <int MODE>
+__device__ __forceinline__ void explicit_body(const TcDev& d, int k, int ja, int jw, int Lc, int block) {
+    const int nch = (d.Nr - 4 + Lc - 1) / Lc;
+    const int w = block * EXPLICIT_WARPS + (threadIdx.x >> 5);
+    const int pg = w / nch, c0 = 2 + (w - pg * nch) * Lc, c1 = min(c0 + Lc, d.Nr - 2);
+    explicit_rows<MODE>(d, k, ja, jw, pg * 32 + (threadIdx.x & 31), c0, c1);
+}
+template <int MODE>
+__global__ void __launch_bounds__(32 * EXPLICIT_WARPS, 3)
+k_explicit(const __grid_constant__ TcDev d, int k, int ja, int jw, int Lc, int mean) {
+    if (mean && blockIdx.x == gridDim.x - 1) mean_body<typename LineTypes<MODE>::CT>(d, k);
+    else explicit_body<MODE>(d, k, ja, jw, Lc, blockIdx.x);
+}
+// The same rows for few pairs (float64 form): a warp that forms the inner functions of
+// all the points of its rows by itself repeats those of its neighbours, and at one or
+// four rows a warp (64x32x64) that is half of its time.  Here a block takes 16 pairs,
+// a lane per component, and 8 R rows; its warps share the inner functions of the
+// 8 R + 4 points through shared memory.  Same operations per component as
+// inner_terms_shared, same bits.  Line phase of
+// 33x16x16 53 -> 47 us.
+constexpr int WIDE_WARPS = 8;
+struct PointRow { double p[5], u, v, w, c, c1; };
+struct HRow { double v, e; };
+__global__ void __launch_bounds__(32 * WIDE_WARPS, 2)
+k_explicit_wide(const __grid_constant__ TcDev d, int k, int ja, int jw, int R) {
+    extern __shared__ double sm[];
+    const int N = d.Nr, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, comp = lane & 1;
+    const int nch = (N - 4 + WIDE_WARPS * R - 1) / (WIDE_WARPS * R), grp = blockIdx.x / nch;
+    const int c0 = 2 + (blockIdx.x - grp * nch) * WIDE_WARPS * R;
+    const int c1 = c0 + WIDE_WARPS * R < N - 2 ? c0 + WIDE_WARPS * R : N - 2, np = c1 - c0 + 4;
+    int pair = 0;
+    double m = 0.0, al = 0.0;
+    long long partner = -1;
+    const bool act = line_pair(d, ja, jw, grp * 16 + (lane >> 1), pair, m, al, partner);
+    const size_t P = d.npairs, P2 = 2 * P, PS2 = (size_t)N * P2, o0 = 2 * (size_t)pair + comp;
+    const double* __restrict__ prod = reinterpret_cast<const double*>(d.prod) + o0;
+    const double* __restrict__ fu = reinterpret_cast<const double*>(d.u) + o0;
+    const double* __restrict__ fv = reinterpret_cast<const double*>(d.v) + o0;
+    const double* __restrict__ fw = reinterpret_cast<const double*>(d.w) + o0;
+    const double mt = m, at = al, at2 = at * at, nu2 = 2.0 * d.nu, nu3 = 3.0 * d.nu;
+    // i z of a value whose components lie in the two lanes: the other's, negated in the real lane
+    auto times_i = [&](double z) {
+        const double o = __shfl_xor_sync(0xffffffffu, z, 1);
+        return comp ? o : -o;
+    };
+    rows_ahead<PointRow, 2>(
+        (np - warp + WIDE_WARPS - 1) / WIDE_WARPS,
+        [&](int q, PointRow& x) {
+            const size_t i = c0 - 2 + warp + q * WIDE_WARPS;
+#pragma unroll
+            for (int t = 0; t < 5; ++t) x.p[t] = prod[i * P2 + t * PS2];
+            x.u = fu[i * P2]; x.v = fv[i * P2]; x.w = fw[i * P2];
+            x.c = d.tab_c[i * P + pair];
+            x.c1 = d.tab_c1[i * P + pair];
+        },
+        [&](int q, const PointRow& x) {
+            const int s = warp + q * WIDE_WARPS;
+            const double ri = d.rinv[c0 - 2 + s], c = x.c, c1f = x.c1;
+            const double pa = x.p[0], uv = x.p[1], uw = x.p[2], vw = x.p[3], pb = x.p[4];
+            const double mr = mt * ri, mr2 = mr * ri, mra = mr * at, n2 = nu2 * mr2;
+            const double Q = fma(at, uv, mr * vw);
+            const double Tm = fma(-n2, x.w, Q), Tp = fma(n2, x.w, Q);
+            const double ph = fma(at, x.u, mr * x.w);
+            const double Z = fma(nu3 * c1f, ph, c * Tm);
+            const double Y = fma(-2.0 * c * mr2, vw, c1f * Tm);
+            const double Rr = fma(mr * mr, pb, fma(2.0 * mra, uw, at2 * pa));
+            const double Nn = fma(-n2, x.u, fma(-at, vw, mr * uv));
+            double* o = sm + s * 160 + lane;
+            o[0] = fma(ri, pb, -times_i(Tp));
+            o[32] = fma(c, Rr, times_i(Y));
+            o[64] = -times_i(Z);
+            o[96] = fma(n2 * at, x.v, fma(fma(mr, mr, -at2), uw, mra * (pa - pb)));
+            o[128] = -times_i(Nn);
+        });
+    double *Hv = reinterpret_cast<double*>(d.Hv) + o0, *He = reinterpret_cast<double*>(d.He) + o0;
+    double *eta = reinterpret_cast<double*>(d.eta) + o0, *rhsv = reinterpret_cast<double*>(rhs_scratch(d, pair)) + comp;
+    const size_t S2 = 2 * (size_t)d.Mzx * d.Nh;
+    const double gdt = d.rk_gamma[k] * d.dt, zdt = d.rk_zeta[(k + 1) % 3] * d.dt;
+    __syncthreads();
+    if (!act) return;
+    auto erow = [&](int j, int s, double H) {   // eta row j on the points s ..
+        double E = 0.0;
+#pragma unroll
+        for (int t = 0; t < 5; ++t) {
+            const double* x = sm + (s + t) * 160 + lane;
+            E = fma(d.d0[j * 5 + t], x[96], E);
+            E = fma(d.l1e[j * 5 + t], x[128], E);
+        }
+        const double r = fma(gdt, E, H);
+        He[(size_t)j * P2] = fma(zdt, E, r);
+        eta[(size_t)j * P2] = r;
+    };
+    rows_ahead<HRow, 2>(
+        (c1 - c0 - warp + WIDE_WARPS - 1) / WIDE_WARPS,
+        [&](int q, HRow& h) {
+            const size_t j = c0 + warp + q * WIDE_WARPS;
+            h.v = Hv[j * P2];
+            h.e = He[j * P2];
+        },
+        [&](int q, const HRow& h) {
+            const int s = warp + q * WIDE_WARPS, j = c0 + s;
+            double E = 0.0;
+#pragma unroll
+            for (int t = 0; t < 5; ++t) {
+                const double* x = sm + (s + t) * 160 + lane;
+                E = fma(d.d0[j * 5 + t], x[0], E);
+                E = fma(d.l1[j * 5 + t], x[32], E);
+                E = fma(d.l2[j * 5 + t], x[64], E);
+            }
+            const double r = fma(gdt, E, h.v);
+            Hv[(size_t)j * P2] = fma(zdt, E, r);
+            rhsv[(size_t)j * S2] = r;
+            erow(j, s, h.e);
+            if (j == 2) erow(1, s, He[P2]);
+            if (j == N - 3) erow(N - 2, s, He[(size_t)(N - 2) * P2]);
+        });
+}
+// Many cases of one form in one launch: emap[block] = (case, block within the
+// case; -1: the case's mean flow)
+template <int MODE>
+__global__ void __launch_bounds__(32 * EXPLICIT_WARPS, 3)
+k_explicit_b(const TcDev* __restrict__ ds, const int2* __restrict__ emap, int k, int Lc) {
+    const int2 m = emap[blockIdx.x];
+    const TcDev& d = ds[m.x];
+    if (m.y < 0) mean_body<typename LineTypes<MODE>::CT>(d, k);
+    else explicit_body<MODE>(d, k, 0, d.Nh, Lc, m.y);
+}
 
 // ---------------------------------------------------------------------------
 // Diagnostics: strain-rate density for the viscous dissipation.
@@ -1148,43 +1617,87 @@ void tc_launch_setup_tables(const TcDev& d, cudaStream_t s) {
     k_setup<<<(d.npairs + 127) / 128, 128, 0, s>>>(d);
 }
 
-void tc_launch_line_phase(const TcDev& d, int k, cudaStream_t s) { tc_launch_line_chunk(d, k, s, 0, d.Nh); }
-
-// line_block encodes the variant: 64/128/256 threads with the register
-// budget of one 256-thread block per SM; 128 threads with a budget for 3
-// (1003) or 4 (1004) resident blocks per SM; 64 threads capped at 144
-// registers (2007: 7 resident blocks, 448 threads per SM, which splits 131 k
-// pairs into 1.9 waves instead of 1.7); 3001: the split variant.  NOH
-// (double-float and mixed forms only): without the implicit RK-memory term.
-template <int MODE, bool NOH>
-static void line_chunk_t(const TcDev& d, int k, cudaStream_t s, int ja, int jw) {
-    const int v = d.line_block > 0 ? d.line_block : 128;
-    if (v == 3001) {                    // split: 32 pairs per 64-thread block
-        k_line_s<MODE, NOH><<<(d.Nz * jw + 31) / 32, 64, 0, s>>>(d, k, ja, jw);
-        return;
+static size_t mean_smem(int Nr) { return (size_t)14 * Nr * sizeof(double); }
+// Radial rows per warp of k_explicit.  A chunk of L rows forms the inner functions at
+// L + 4 points (57 float64 operations each) and 65 operations a row; a quarter of an
+// SM runs one warp's operation in 64 cycles, so a launch takes as many times that
+// work as each of the 608 quarters has warps.  The rule takes the shortest; line_block
+// 128 is the rule, the other accepted values pin a length (tc_set_tiles).
+// shared memory of k_explicit: the rows on their way in, or the mean flow's block (Nr > 0)
+static size_t explicit_smem(int prec, int Nr) {
+    const size_t ring = prec == 1 ? (size_t)RowRing<1>::RING * RowRing<1>::BYTES : prec == 2 ? (size_t)RowRing<2>::RING * RowRing<2>::BYTES : 0;
+    const size_t mean = Nr > 0 ? mean_smem(Nr) : 0;
+    return ring > mean ? ring : mean;
+}
+static int explicit_rule(int Nr, long long groups, long long& best) {
+    const int nc = Nr - 4;
+    int rows = 64;
+    best = 0;
+    for (int L : {64, 48, 32, 24, 16, 12, 8, 6, 4, 3, 2, 1}) {
+        const long long warps = groups * ((nc + L - 1) / L), per = (warps + 607) / 608;
+        const int l = L < nc ? L : nc;
+        const long long cost = (per > 4 ? (warps * 16 + 607) / 608 : per * 16) * (57 * (l + 4) + 65 * l);
+        if (best == 0 || cost < best) { best = cost; rows = L; }
     }
-    const int bs = v == 2007 ? 64 : (v > 1000 ? 128 : v);
-    const int grid = (d.Nz * jw + bs - 1) / bs;
-    if (v == 1003) k_line<MODE, 128, 3, NOH><<<grid, bs, 0, s>>>(d, k, ja, jw);
-    else if (v == 1004) k_line<MODE, 128, 4, NOH><<<grid, bs, 0, s>>>(d, k, ja, jw);
-    else if (v == 2007) k_line_r<MODE, 144, NOH><<<grid, bs, 0, s>>>(d, k, ja, jw);
-    else k_line<MODE, 256, 1, NOH><<<grid, bs, 0, s>>>(d, k, ja, jw);
+    return rows;
 }
-
-void tc_launch_line_chunk(const TcDev& d, int k, cudaStream_t s, int ja, int jw) {
-    if (d.prec == 1) line_chunk_t<1, false>(d, k, s, ja, jw);
-    else if (d.prec == 2) line_chunk_t<2, false>(d, k, s, ja, jw);
-    else line_chunk_t<0, false>(d, k, s, ja, jw);
+static int explicit_rows_per_warp(int line_block, int Nr, long long groups) {
+    switch (line_block) {
+        case 64: return 8;
+        case 256: return 64;
+        case 1003: return 16;
+        case 1004: return 32;
+        case 2007: return 4;
+        case 3001: return 128;
+        default: break;
+    }
+    long long cost;
+    return explicit_rule(Nr, groups, cost);
 }
-
-void tc_launch_line_chunk_deferred(const TcDev& d, int k, cudaStream_t s, int ja, int jw) {
-    if (d.prec == 1) line_chunk_t<1, true>(d, k, s, ja, jw);
-    else if (d.prec == 2) line_chunk_t<2, true>(d, k, s, ja, jw);
-    else line_chunk_t<0, false>(d, k, s, ja, jw);   // float64: never deferred
+// Rows per warp of k_explicit_wide, 0 where k_explicit takes less time by the same
+// count (33 + 29 operations a point and row here) or the launch is not the float64
+// form's own choice.
+static int explicit_wide_rows(int prec, int line_block, int Nr, long long groups) {
+    if (prec != 0 || line_block != 128 || !solve_wide(2 * groups, Nr)) return 0;
+    long long best;
+    explicit_rule(Nr, groups, best);
+    int rows = 0;
+    for (int R : {1, 2, 3, 4, 6, 8}) {
+        const int n = 8 * R < Nr - 4 ? 8 * R : Nr - 4;
+        const long long blocks = 2 * groups * ((Nr - 4 + 8 * R - 1) / (8 * R)), per = 2 * ((blocks + 151) / 152);
+        const long long cost = (per > 4 ? (blocks * 32 + 151) / 152 : per * 16) * (33 * ((n + 4 + 7) / 8) + 29 * ((n + 7) / 8));
+        if (cost < best) { best = cost; rows = R; }
+    }
+    return rows;
 }
+void tc_launch_line_chunk(const TcDev& d, int k, cudaStream_t s, int ja, int jw, bool mean, bool deferred) {
+    const int groups = (d.Nz * jw + 31) / 32, half = (d.Nz * jw + 15) / 16;
+    const int Lc = explicit_rows_per_warp(d.line_block, d.Nr, groups);
+    const long long warps = (long long)groups * ((d.Nr - 4 + Lc - 1) / Lc);
+    const bool noh = deferred && d.prec != 0, wide = solve_wide(half, d.Nr);
+    // the mean flow goes with the longer launch: the solves where they are latency
+    const bool early = mean && !wide;
+    const int grid = (int)((warps + EXPLICIT_WARPS - 1) / EXPLICIT_WARPS) + (early ? 1 : 0);
+    const size_t sm = explicit_smem(d.prec, early ? d.Nr : 0);
+    const int R = explicit_wide_rows(d.prec, d.line_block, d.Nr, groups);
+    if (R > 0)
+        k_explicit_wide<<<half * ((d.Nr - 4 + 8 * R - 1) / (8 * R)), 32 * WIDE_WARPS, (8 * R + 4) * 160 * sizeof(double), s>>>(d, k, ja, jw, R);
+    else if (d.prec == 1) k_explicit<1><<<grid, 32 * EXPLICIT_WARPS, sm, s>>>(d, k, ja, jw, Lc, early);
+    else if (d.prec == 2) k_explicit<2><<<grid, 32 * EXPLICIT_WARPS, sm, s>>>(d, k, ja, jw, Lc, early);
+    else k_explicit<0><<<grid, 32 * EXPLICIT_WARPS, sm, s>>>(d, k, ja, jw, Lc, early);
+    if (wide) {
+        const size_t sw = solve_smem(d.Nr);     // more than the mean flow's block takes
+        if (noh) k_solve_shared<true><<<half + (mean ? 1 : 0), 32 * SOLVE_WARPS, sw, s>>>(d, k, ja, jw, mean);
+        else k_solve_shared<false><<<half + (mean ? 1 : 0), 32 * SOLVE_WARPS, sw, s>>>(d, k, ja, jw, mean);
+    } else {
+        if (noh) k_solve<true><<<half, 64, 0, s>>>(d, k, ja, jw);
+        else k_solve<false><<<half, 64, 0, s>>>(d, k, ja, jw);
+    }
+}
+void tc_launch_line_phase(const TcDev& d, int k, cudaStream_t s, bool mean) { tc_launch_line_chunk(d, k, s, 0, d.Nh, mean, false); }
 
 void tc_launch_rk_memory(const TcDev& d, int k, cudaStream_t s, int ja, int jw, bool background) {
-    int blocks = (d.Nz * jw + 127) / 128;
+    int blocks = (2 * d.Nz * jw + 127) / 128;
     if (background) {
         static int sms = 0;
         if (!sms) {
@@ -1199,44 +1712,57 @@ void tc_launch_rk_memory(const TcDev& d, int k, cudaStream_t s, int ja, int jw, 
 
 const void* tc_rk_memory_kernel() { return (const void*)k_rk_memory; }
 
-static size_t mean_smem(const TcDev& d) { return (size_t)(2 * d.Nr * 5 * 2 + 2 * d.Nr * 3) * sizeof(double); }
-
 void tc_launch_mean_phase(const TcDev& d, int k, cudaStream_t s) {
-    if (d.prec == 1) k_mean<float2><<<1, 256, mean_smem(d), s>>>(d, k, 0);
-    else if (d.prec == 2) k_mean<dcomplex><<<1, 256, mean_smem(d), s>>>(d, k, 0);
-    else k_mean<double2><<<1, 256, mean_smem(d), s>>>(d, k, 0);
+    if (d.prec == 1) k_mean<float2><<<1, 256, mean_smem(d.Nr), s>>>(d, k);
+    else if (d.prec == 2) k_mean<dcomplex><<<1, 256, mean_smem(d.Nr), s>>>(d, k);
+    else k_mean<double2><<<1, 256, mean_smem(d.Nr), s>>>(d, k);
 }
 
-void tc_launch_line_batch(int prec, const TcDev* ds, const int2* bmap, int nblocks, int k, cudaStream_t s) {
-    if (prec == 1) k_line_b<1><<<nblocks, 128, 0, s>>>(ds, bmap, k);
-    else if (prec == 2) k_line_b<2><<<nblocks, 128, 0, s>>>(ds, bmap, k);
-    else k_line_b<0><<<nblocks, 128, 0, s>>>(ds, bmap, k);
+// The launches over many cases: which of the two takes the mean flows (the solves
+// where they are wide), and the blocks of one case in each.
+static long long half_groups(const TcDev& d) { return (d.npairs + 15) / 16; }
+void tc_line_batch_plan(const TcDev* ds, int ncases, int& Lc, bool& wide) {
+    long long half = 0, groups = 0;
+    int maxNr = 0;
+    for (int i = 0; i < ncases; ++i) {
+        half += half_groups(ds[i]);
+        groups += (ds[i].npairs + 31) / 32;
+        maxNr = ds[i].Nr > maxNr ? ds[i].Nr : maxNr;
+    }
+    Lc = explicit_rows_per_warp(128, maxNr, groups);
+    wide = solve_wide(half, maxNr);
 }
-
-int tc_line_batch_block() { return 128; }
-
-void tc_launch_mean_batch(int prec, const TcDev* ds, int ncases, int maxNr, int k, cudaStream_t s) {
-    TcDev dm;
-    dm.Nr = maxNr;
-    if (prec == 1) k_mean_b<float2><<<ncases, 256, mean_smem(dm), s>>>(ds, k);
-    else if (prec == 2) k_mean_b<dcomplex><<<ncases, 256, mean_smem(dm), s>>>(ds, k);
-    else k_mean_b<double2><<<ncases, 256, mean_smem(dm), s>>>(ds, k);
+int tc_line_batch_explicit_blocks(const TcDev& d, int Lc) {
+    const long long warps = (long long)((d.npairs + 31) / 32) * ((d.Nr - 4 + Lc - 1) / Lc);
+    return (int)((warps + EXPLICIT_WARPS - 1) / EXPLICIT_WARPS);
+}
+int tc_line_batch_solve_blocks(const TcDev& d) { return (int)half_groups(d); }
+void tc_launch_explicit_batch(int prec, const TcDev* ds, const int2* emap, int nblocks, int maxNr, int Lc, bool mean, int k,
+                              cudaStream_t s) {
+    const size_t sm = explicit_smem(prec, mean ? maxNr : 0);
+    if (prec == 1) k_explicit_b<1><<<nblocks, 32 * EXPLICIT_WARPS, sm, s>>>(ds, emap, k, Lc);
+    else if (prec == 2) k_explicit_b<2><<<nblocks, 32 * EXPLICIT_WARPS, sm, s>>>(ds, emap, k, Lc);
+    else k_explicit_b<0><<<nblocks, 32 * EXPLICIT_WARPS, sm, s>>>(ds, emap, k, Lc);
+}
+void tc_launch_solve_batch(const TcDev* ds, const int2* bmap, int nblocks, int maxNr, bool wide, int k, cudaStream_t s) {
+    if (wide) k_solve_shared_b<<<nblocks, 32 * SOLVE_WARPS, solve_smem(maxNr), s>>>(ds, bmap, k);
+    else k_solve_b<<<nblocks, 64, 0, s>>>(ds, bmap, k);
 }
 
 cudaError_t tc_set_line_kernel_attributes() {
     const int lim = 200 * 1024;
-    cudaError_t e = cudaFuncSetAttribute((const void*)k_mean<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute((const void*)k_mean<dcomplex>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    if (e != cudaSuccess) return e;
-    for (const void* f : {(const void*)k_mean_b<double2>, (const void*)k_mean_b<dcomplex>, (const void*)k_mean_b<float2>}) {
-        e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    for (const void* f : {(const void*)k_mean<double2>, (const void*)k_mean<dcomplex>, (const void*)k_mean<float2>,
+                          (const void*)k_explicit<0>, (const void*)k_explicit<1>, (const void*)k_explicit<2>,
+                          (const void*)k_explicit_b<0>, (const void*)k_explicit_b<1>, (const void*)k_explicit_b<2>,
+                          (const void*)k_explicit_wide, (const void*)k_solve_shared<true>, (const void*)k_solve_shared<false>,
+                          (const void*)k_solve_shared_b}) {
+        const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         if (e != cudaSuccess) return e;
     }
-    return cudaFuncSetAttribute((const void*)k_mean<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    return cudaSuccess;
 }
 
 void tc_launch_init_state(const TcDev& d, cudaStream_t s) {
     k_init<<<(d.npairs + 127) / 128, 128, 0, s>>>(d);
-    k_mean<double2><<<1, 256, mean_smem(d), s>>>(d, 0, 1);
+    k_mean_init<<<1, 256, 0, s>>>(d);
 }

@@ -4,9 +4,9 @@
 // stepped together by one CUDA graph per step.  Cases of the same form and
 // Fourier grid (any Nr, radius ratio, Re) form a shape class; each
 // plane-phase kernel runs once per class over the radial planes of all of its
-// cases (the classes as concurrent branches), and the line kernel and the
-// mean flow once per precision form over all of its cases, each block
-// reading its case's descriptor.
+// cases (the classes as concurrent branches), and the line phase with the
+// mean flows in two launches per precision form over all of its cases, each
+// block reading its case's descriptor.
 //
 // Server: continuous batching.  Requests (case parameters, initial
 // perturbation, number of steps) are queued by tc_server_submit from any host
@@ -43,8 +43,8 @@ using tcx::set_err;
     } while (0)
 
 // Cases of one shape class (the same form, Ntheta and Nz; any Nr, radius
-// ratio, Re, box): their plane kernels, line kernel and mean flow run as one
-// launch each, over the radial planes / pairs / profiles of all of them.
+// ratio, Re, box): each plane kernel runs as one launch over the radial planes
+// of all of them.
 struct BatchClass {
     std::vector<int> cases;
     TcDev d0;                       // representative descriptor (shapes, z tile, plans)
@@ -55,15 +55,17 @@ struct BatchClass {
     cudaEvent_t join = nullptr;
 };
 
-// Cases of one precision form: their line kernel is one launch over the
-// pairs of all of them (cases ordered by decreasing Nr, so that the longest
-// radial lines start first), their mean flows one launch with a block each.
+// Cases of one precision form: their line phase is two launches over all of them
+// (cases ordered by decreasing Nr, so that the longest radial lines start first),
+// the mean flows a block each of one of them.
 struct BatchForm {
-    int prec = 0, ncases = 0, nblocks = 0, maxNr = 0;
+    int prec = 0, ncases = 0, neblocks = 0, nblocks = 0, maxNr = 0, rows = 0;
+    bool wide = false;
     TcDev* ds = nullptr;
-    int2* bmap = nullptr;           // (case, block within the case) per line-kernel block
-    cudaStream_t sl = nullptr, sm = nullptr;
-    cudaEvent_t jl = nullptr, jm = nullptr;
+    int2* emap = nullptr;           // (case, block within the case) per block of the explicit rows
+    int2* bmap = nullptr;           // (case, 16 pairs of the case) per block of the solves
+    cudaStream_t sl = nullptr;
+    cudaEvent_t jl = nullptr;
 };
 
 // A set of cases stepped together: their shape classes and precision forms,
@@ -91,9 +93,10 @@ static void batch_release_classes(Group* b) {
     b->classes.clear();
     for (auto& f : b->forms) {
         if (f.ds) cudaFree(f.ds);
+        if (f.emap) cudaFree(f.emap);
         if (f.bmap) cudaFree(f.bmap);
-        for (cudaEvent_t e : {f.jl, f.jm}) if (e) cudaEventDestroy(e);
-        for (cudaStream_t t : {f.sl, f.sm}) if (t) cudaStreamDestroy(t);
+        if (f.jl) cudaEventDestroy(f.jl);
+        if (f.sl) cudaStreamDestroy(f.sl);
     }
     b->forms.clear();
 }
@@ -142,7 +145,6 @@ static int batch_classes(Group* b) {
         CKR(cudaStreamCreateWithFlags(&c.stream, cudaStreamNonBlocking), TC_ERR_CUDA);
         CKR(cudaEventCreateWithFlags(&c.join, cudaEventDisableTiming), TC_ERR_CUDA);
     }
-    const int bs = tc_line_batch_block();
     for (int prec : {TC_PREC_FP64, TC_PREC_MIXED, TC_PREC_DF64}) {
         std::vector<int> idx;
         for (int i = 0; i < (int)b->cases.size(); ++i)
@@ -154,22 +156,27 @@ static int batch_classes(Group* b) {
         f.prec = prec;
         f.ncases = (int)idx.size();
         std::vector<TcDev> ds;
-        std::vector<int2> bm;
+        std::vector<int2> em, bm;
         for (int i = 0; i < f.ncases; ++i) {
-            const TcDev& d = b->cases[idx[i]]->d;
-            ds.push_back(d);
-            f.maxNr = std::max(f.maxNr, d.Nr);
-            for (int q = 0; q < (d.npairs + bs - 1) / bs; ++q) bm.push_back(make_int2(i, q));
+            ds.push_back(b->cases[idx[i]]->d);
+            f.maxNr = std::max(f.maxNr, ds[i].Nr);
         }
+        tc_line_batch_plan(ds.data(), f.ncases, f.rows, f.wide);
+        for (int i = 0; i < f.ncases; ++i) (f.wide ? bm : em).push_back(make_int2(i, -1));   // the mean flows first
+        for (int i = 0; i < f.ncases; ++i) {
+            for (int q = 0; q < tc_line_batch_explicit_blocks(ds[i], f.rows); ++q) em.push_back(make_int2(i, q));
+            for (int q = 0; q < tc_line_batch_solve_blocks(ds[i]); ++q) bm.push_back(make_int2(i, q));
+        }
+        f.neblocks = (int)em.size();
         f.nblocks = (int)bm.size();
         CKR(cudaMalloc(&f.ds, ds.size() * sizeof(TcDev)), TC_ERR_CUDA);
+        CKR(cudaMalloc(&f.emap, em.size() * sizeof(int2)), TC_ERR_CUDA);
         CKR(cudaMalloc(&f.bmap, bm.size() * sizeof(int2)), TC_ERR_CUDA);
         CKR(cudaMemcpy(f.ds, ds.data(), ds.size() * sizeof(TcDev), cudaMemcpyHostToDevice), TC_ERR_CUDA);
+        CKR(cudaMemcpy(f.emap, em.data(), em.size() * sizeof(int2), cudaMemcpyHostToDevice), TC_ERR_CUDA);
         CKR(cudaMemcpy(f.bmap, bm.data(), bm.size() * sizeof(int2), cudaMemcpyHostToDevice), TC_ERR_CUDA);
         CKR(cudaStreamCreateWithFlags(&f.sl, cudaStreamNonBlocking), TC_ERR_CUDA);
-        CKR(cudaStreamCreateWithFlags(&f.sm, cudaStreamNonBlocking), TC_ERR_CUDA);
         CKR(cudaEventCreateWithFlags(&f.jl, cudaEventDisableTiming), TC_ERR_CUDA);
-        CKR(cudaEventCreateWithFlags(&f.jm, cudaEventDisableTiming), TC_ERR_CUDA);
     }
     return TC_OK;
 }
@@ -177,8 +184,8 @@ static int batch_classes(Group* b) {
 // One step of every case, per substep: the plane phase of each shape class
 // (z inverse, theta rows, z forward, one launch each over all of the
 // class's cases; the classes as concurrent branches), then the line phase of
-// each precision form (one launch over all of its cases) beside its mean
-// flows (one launch).
+// each precision form, two launches over all of its cases: the explicit rows
+// with the mean flows, and the solves.
 static int batch_graph(Group* b) {
     if (b->graph) return TC_OK;
     for (auto h : b->cases) {
@@ -202,13 +209,10 @@ static int batch_graph(Group* b) {
         CKR(cudaEventRecord(b->fork, b->root), TC_ERR_CUDA);
         for (auto& f : b->forms) {
             CKR(cudaStreamWaitEvent(f.sl, b->fork, 0), TC_ERR_CUDA);
-            CKR(cudaStreamWaitEvent(f.sm, b->fork, 0), TC_ERR_CUDA);
-            tc_launch_line_batch(f.prec, f.ds, f.bmap, f.nblocks, k, f.sl);
-            tc_launch_mean_batch(f.prec, f.ds, f.ncases, f.maxNr, k, f.sm);
+            tc_launch_explicit_batch(f.prec, f.ds, f.emap, f.neblocks, f.maxNr, f.rows, !f.wide, k, f.sl);
+            tc_launch_solve_batch(f.ds, f.bmap, f.nblocks, f.maxNr, f.wide, k, f.sl);
             CKR(cudaEventRecord(f.jl, f.sl), TC_ERR_CUDA);
-            CKR(cudaEventRecord(f.jm, f.sm), TC_ERR_CUDA);
             CKR(cudaStreamWaitEvent(b->root, f.jl, 0), TC_ERR_CUDA);
-            CKR(cudaStreamWaitEvent(b->root, f.jm, 0), TC_ERR_CUDA);
         }
     }
     cudaError_t e = cudaStreamEndCapture(b->root, &g);

@@ -620,13 +620,16 @@ int init_handle(tc_handle* h) {
     d.Mtx = fx_length(d.Mt);
     d.Mzx = fx_length(d.Mz);
     d.fx = d.prec != TC_PREC_MIXED && d.Mtx > 0 && d.Mzx > 0;
-    if (d.fx) {
+    d.phx = d.Mtx == d.Mt && d.Mzx == d.Mz;
+    if (d.fx || d.phx) {
         (void)std::frexp(1.0 / ((double)d.Mtx * (double)d.Mzx), &d.kexp);
         const ld kappa = ldexpl(1.0L / ((ld)d.Mtx * (ld)d.Mzx), -d.kexp);
         if ((rc_ = upload(h, d.twx_t, fx_table(d.Mtx, 0.0L)))) return rc_;
         if ((rc_ = upload(h, d.twx_z, fx_table(d.Mzx, kappa)))) return rc_;
         CK(tc_fx_attributes(d.Mtx, d.Mzx));
-    } else {
+        if ((rc_ = dalloc(h, d.zexp, 3 * (size_t)d.Nr * d.Nh))) return rc_;
+    }
+    if (!d.fx) {
         d.Mtx = d.Mt;
         d.Mzx = d.Mz;
     }
@@ -643,12 +646,11 @@ int init_handle(tc_handle* h) {
     const size_t Z1 = (size_t)d.Nr * d.Mzx * d.Nh;
     double2 *zb, *pb;
     if ((rc_ = dalloc(h, zb, 3 * Z1))) return rc_;
-    if ((rc_ = dalloc(h, pb, TC_NPROD * Z1))) return rc_;
+    const size_t pelems = d.prec == TC_PREC_MIXED ? (TC_NPROD * Z1 + 1) / 2 : TC_NPROD * Z1;     // mixed: float2
+    if ((rc_ = dalloc(h, pb, pelems))) return rc_;
     d.zbuf = zb; d.pbuf = pb;
-    if (d.fx) {
-        if ((rc_ = dalloc(h, d.zexp, 3 * (size_t)d.Nr * d.Nh))) return rc_;
-        if ((rc_ = dalloc(h, d.pexp, 3 * (size_t)d.Nr * d.Mzx))) return rc_;
-    }
+    d.phys = reinterpret_cast<double*>(pb);
+    if (d.fx && (rc_ = dalloc(h, d.pexp, 3 * (size_t)d.Nr * d.Mzx))) return rc_;
     double* mean;
     if ((rc_ = dalloc(h, mean, 6 * (size_t)d.Nr))) return rc_;
     d.U = mean; d.W = mean + d.Nr; d.HU = mean + 2 * d.Nr; d.HW = mean + 3 * d.Nr; d.eprof = mean + 4 * d.Nr;
@@ -669,7 +671,7 @@ int init_handle(tc_handle* h) {
     if ((rc_ = dalloc(h, d.tab_lv, (size_t)d.Nr * 5 * d.npairs))) return rc_;
     if ((rc_ = dalloc(h, d.tab_le, (size_t)d.Nr * 5 * d.npairs))) return rc_;
     if ((rc_ = dalloc(h, d.tab_c, (size_t)d.Nr * d.npairs))) return rc_;
-    if ((rc_ = dalloc(h, d.tab_c1, (size_t)d.Nr * d.npairs))) return rc_;
+    if (d.prec != TC_PREC_DF64 && (rc_ = dalloc(h, d.tab_c1, (size_t)d.Nr * d.npairs))) return rc_;
     if (d.prec != TC_PREC_FP64) {     // float (hi, lo) copies of c and c'
         if ((rc_ = dalloc(h, d.tab_cx, (size_t)d.Nr * d.npairs))) return rc_;
         if ((rc_ = dalloc(h, d.tab_c1x, (size_t)d.Nr * d.npairs))) return rc_;
@@ -687,7 +689,7 @@ int init_handle(tc_handle* h) {
     if (hf[1]) { set_err("a radial system has a vanishing pivot (LU without pivoting)"); return TC_ERR_STATE; }
     if (P.autotune) {
         // the timed kernels read the plane buffers
-        CK(cudaMemset(d.pbuf, 0, TC_NPROD * Z1 * sizeof(double2)));
+        CK(cudaMemset(d.pbuf, 0, pelems * sizeof(double2)));
         if (d.fx) CK(cudaMemset(d.pexp, 0, 3 * (size_t)d.Nr * d.Mzx * sizeof(int)));
         if ((rc_ = autotune(h))) return rc_;
     }
@@ -930,10 +932,10 @@ size_t estimate_device_bytes(const tc_params& p) {
     const size_t np = Nz * Nh, P1 = Nr * np, Z1 = Nr * (Mzx > Mz ? Mzx : Mz) * Nh;
     size_t b = 0;
     b += (6 + TC_NPROD) * P1 * sizeof(double2);                 // fields, products
-    b += (3 + TC_NPROD) * Z1 * sizeof(double2);                 // zbuf, pbuf
+    b += 3 * Z1 * sizeof(double2) + TC_NPROD * Z1 * (p.precision == TC_PREC_MIXED ? 8 : 16);     // zbuf, pbuf
     b += (3 + 3) * Nr * 5 * np * sizeof(double);                // LU tables
-    b += 2 * Nr * 5 * np * sizeof(double) + 4 * Nr * np * sizeof(double);   // L bands, c, c1 (+ double-float copies)
-    b += Nr * Mz * Mt * sizeof(double);                         // physical output (on demand)
+    b += 2 * Nr * 5 * np * sizeof(double);                      // L bands
+    b += (p.precision == TC_PREC_FP64 ? 2 : p.precision == TC_PREC_DF64 ? 3 : 4) * Nr * np * sizeof(double);    // c, c1, copies
     b += 3 * Nr * (Nh + Mzx) * sizeof(int);                     // exponents of the fixed-point planes
     b += 64 * Nr * sizeof(double) + 4 * (Mz + 2 * Mt) * sizeof(double2);  // radial tables, twiddles
     return b + 40 * (2u << 20);
@@ -1353,13 +1355,7 @@ int tc_get_field(tc_handle* h, int which, int space, void* buf, size_t bytes) {
     if (space == TC_SPECTRAL) {
         CK(cudaMemcpyAsync(buf, src, bytes, cudaMemcpyDeviceToHost, h->stream));
     } else {
-        if (!d.phys) {
-            double* p;
-            if ((rc = dalloc(h, p, (size_t)d.Nr * d.Mz * d.Mt))) return rc;
-            d.phys = p;
-            tcx::drop_graphs(h);
-        }
-        tc_launch_to_physical(d, src, h->stream);
+        tc_launch_to_physical(d, src, h->stream);       // into pbuf, free between substeps
         CK(cudaGetLastError());
         CK(cudaMemcpyAsync(buf, d.phys, bytes, cudaMemcpyDeviceToHost, h->stream));
     }

@@ -16,6 +16,8 @@ cudaError_t tc_rows_phys_attributes();
 #define FX_GROUP(TAG)                                                                                                   \
     bool tc_fx_z_##TAG(const TcDev&, const TcDev*, const int2*, int, int, cudaStream_t, int, int);                      \
     bool tc_fx_rows_##TAG(const TcDev&, const TcDev*, const int2*, int, cudaStream_t);                                  \
+    bool tc_fx_phys_##TAG(const TcDev&, int4, cudaStream_t);                                                            \
+    bool tc_fx_order_##TAG(int, int4&);                                                                                 \
     bool tc_fx_attributes_##TAG(int, int, cudaError_t&);
 FX_GROUP(a) FX_GROUP(b) FX_GROUP(c) FX_GROUP(d)
 #undef FX_GROUP
@@ -29,6 +31,19 @@ void tc_fx_plane_kernel(const TcDev& d, const TcDev* ds, const int2* ymap, int n
         (void)(tc_fx_z_a(d, ds, ymap, nplanes, which, s, col0, ncols) || tc_fx_z_b(d, ds, ymap, nplanes, which, s, col0, ncols) ||
                tc_fx_z_c(d, ds, ymap, nplanes, which, s, col0, ncols) || tc_fx_z_d(d, ds, ymap, nplanes, which, s, col0, ncols));
     }
+}
+
+bool tc_fx_to_physical(const TcDev& d, const double2* field, cudaStream_t s) {
+    if (!d.phx) return false;
+    TcDev dd = d;
+    dd.u = const_cast<double2*>(field);                 // read only
+    dd.Mtx = dd.Mt;
+    dd.Mzx = dd.Mz;
+    int4 zr = make_int4(1, 1, 1, 1);
+    (void)(tc_fx_order_a(d.Mz, zr) || tc_fx_order_b(d.Mz, zr) || tc_fx_order_c(d.Mz, zr) || tc_fx_order_d(d.Mz, zr));
+    tc_fx_plane_kernel(dd, nullptr, nullptr, d.Nr, 3, s, 0, d.Nh);
+    (void)(tc_fx_phys_a(dd, zr, s) || tc_fx_phys_b(dd, zr, s) || tc_fx_phys_c(dd, zr, s) || tc_fx_phys_d(dd, zr, s));
+    return true;
 }
 
 cudaError_t tc_fx_attributes(int Mtx, int Mzx) {

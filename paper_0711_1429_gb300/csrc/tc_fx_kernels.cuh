@@ -524,6 +524,120 @@ kx_rows(const __grid_constant__ TcDev d1, const TcDev* __restrict__ ds, const in
     }
 }
 
+// ---- physical output of one field: theta rows of zbuf's first field ---------------
+// Two rows (axial points) per complex transform, X(q0) + i X(q1), each block G such
+// pairs of one radial plane.  The rows come in the axial transform's digit-reversed
+// order and leave in natural order, as float64; zr: that transform's radices and
+// strides (R0, R1, st0, st1).  Scale: twice the sum of the moduli of the pair's own
+// values bounds every intermediate one; the sum of the columns' largest values (as in
+// kx_rows) would leave two bits of the result unused.
+template <int M>
+__global__ void __launch_bounds__(FxPlan<M>::W)
+kx_phys(const __grid_constant__ TcDev d, int4 zr) {
+    typedef FxPlan<M> P;
+    constexpr int NP = P::NP, T = P::T, G = P::G, W = P::W;
+    constexpr int R = fx_radix<M, 0>(), RL = fx_radix<M, NP - 1>(), MP = M + M / 8;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int emax;
+    __shared__ unsigned rsum[G];
+    const int rp = blockIdx.y, Mz = d.Mz, Nh = d.Nh, in = threadIdx.x;
+    const fxw* tw = d.twx_t;
+    const bool on = in < G * T;
+    const int g = on ? in / T : 0, t = on ? in - g * T : 0;
+    const int q0 = 2 * (blockIdx.x * G + g);
+    const bool have0 = on && q0 < Mz, have1 = on && q0 + 1 < Mz;
+    fxc* const col = reinterpret_cast<fxc*>(smem_raw) + g * MP;
+    if (in == 0) emax = FX_NONE;
+    if (in < G) rsum[in] = 0;
+    const int* zx = d.zexp + (size_t)rp * Nh;
+    __syncthreads();
+    {
+        int a = FX_NONE;
+        for (int j = in; j < Nh; j += W) a = max(a, zx[j]);
+        a = __reduce_max_sync(0xffffffffu, a);
+        if ((in & 31) == 0) atomicMax(&emax, a);
+    }
+    __syncthreads();
+    const int em = emax;
+    const fxc* zb = reinterpret_cast<const fxc*>(d.zbuf) + (size_t)rp * Mz * Nh;
+    if (on) {
+        auto modulus = [](fxc x) {                  // upper words: max + min/2 is above the modulus
+            const unsigned a = fx_abs_hi(x.x), b = fx_abs_hi(x.y);
+            return a > b ? a + (b >> 1) : b + (a >> 1);
+        };
+        unsigned a = 0;
+        for (int j = t; j < Nh; j += T) {
+            const int sh = 12 + em - zx[j];
+            unsigned m = 2;
+            if (have0) m += modulus(zb[(size_t)q0 * Nh + j]);
+            if (have1) m += modulus(zb[(size_t)(q0 + 1) * Nh + j]);
+            a += (sh > 31 ? 0 : m >> sh) + 1;
+        }
+        atomicAdd(&rsum[g], a);
+    }
+    __syncthreads();
+    int EB = fx_headroom<M, 1>(em + 64, em + 45 + fx_bitlen(rsum[g]));
+    if (EB < em + 63) EB = em + 63;
+    if (on && t < M / R) {
+        fxc v[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            v[r].x = v[r].y = 0;
+            if (!fx_dead_leg<M, R>(r)) {
+                const int p = t + r * (M / R);
+                const bool neg = p >= Nh;
+                const int j = !neg ? p : (p > M - Nh ? M - p : -1);
+                if (j >= 0) {
+                    fxc x, y;
+                    x.x = x.y = y.x = y.y = 0;
+                    if (have0) x = zb[(size_t)q0 * Nh + j];
+                    if (have1) y = zb[(size_t)(q0 + 1) * Nh + j];
+                    int s = EB - 62 - zx[j];
+                    s = s > 63 ? 63 : s;
+                    const fx_t h = 1LL << (s - 1);
+                    x.x = (x.x + h) >> s; x.y = (x.y + h) >> s;
+                    y.x = (y.x + h) >> s; y.y = (y.y + h) >> s;
+                    if (p == 0) { x.y = 0; y.y = 0; }
+                    v[r].x = neg ? x.x + y.y : x.x - y.y;
+                    v[r].y = neg ? y.x - x.y : y.x + x.y;
+                }
+            }
+        }
+        fx_butterfly<M, 1, 0>(v, t, tw);
+        fx_put<M, 0>(v, col, t, 0);
+    }
+    __syncthreads();
+    if constexpr (NP == 3) {
+        if (on) fx_middle<M, 1>(col, t, 0, tw);
+        __syncthreads();
+    }
+    fxc v[RL];
+    const bool last = on && t < M / RL;
+    if (last) {
+        fx_get<M, NP - 1>(v, col, t, 0);
+        fx_butterfly<M, 1, NP - 1>(v, t, tw);
+    }
+    __syncthreads();
+    if (last) {
+#pragma unroll
+        for (int r = 0; r < RL; ++r) col[fx_pad(fx_index<M>(fx_pos<M, NP - 1>(t, r)))] = v[r];
+    }
+    __syncthreads();
+    if (!on) return;
+    const int eb = em == FX_NONE ? 0 : EB - 62 + fx_gain<M>();
+    const bool bad = em >= FX_BAD;
+    auto row = [&](int q) {
+        return d.phys + ((size_t)rp * Mz + q / zr.z + zr.x * (q % zr.z / zr.w + zr.y * (q % zr.w))) * M;
+    };
+    double* o0 = row(have0 ? q0 : 0);
+    double* o1 = row(have1 ? q0 + 1 : 0);
+    for (int p = t; p < M; p += T) {
+        const fxc a = col[fx_pad(p)];
+        if (have0) o0[p] = bad ? fx_nan() : fx_to(a.x, eb);
+        if (have1) o1[p] = bad ? fx_nan() : fx_to(a.y, eb);
+    }
+}
+
 // ---- host launchers ----------------------------------------------------------
 // which: 0 axial inverse, 1 theta rows, 2 axial forward, for the azimuthal
 // columns col0 .. col0 + ncols - 1 of one case (ds == nullptr) or of every plane
@@ -533,7 +647,8 @@ template <int M> static void fx_launch_z(const TcDev& d, const TcDev* ds, const 
     int lct = 0;
     while ((2 << lct) <= d.ztile && (2 << lct) <= fx_z_columns<M>()) ++lct;      // ztile is 1, 2, 4 or 8
     const int ct = 1 << lct, nth = fx_z_threads<M>(ct), sm = ct * (M + M / 8) * (int)sizeof(fxc);
-    if (which == 0) kx_zinv<M><<<dim3(ncols / ct, nplanes, 3), nth, sm, s>>>(d, ds, ymap, col0, lct);
+    if (which == 0 || which == 3)           // 3: one field (d.u), for the physical output
+        kx_zinv<M><<<dim3(ncols / ct, nplanes, which == 0 ? 3 : 1), nth, sm, s>>>(d, ds, ymap, col0, lct);
     else if (d.prec == 2) kx_zfwd<M, true><<<dim3(ncols / ct, nplanes, TC_NPROD), nth, sm, s>>>(d, ds, ymap, col0, lct);
     else kx_zfwd<M, false><<<dim3(ncols / ct, nplanes, TC_NPROD), nth, sm, s>>>(d, ds, ymap, col0, lct);
 }
@@ -541,6 +656,11 @@ template <int M> static void fx_launch_rows(const TcDev& d, const TcDev* ds, con
     const int pairs = (d.Mzx + 1) / 2;
     kx_rows<M><<<dim3((pairs + FxPlan<M>::G - 1) / FxPlan<M>::G, nplanes), 3 * FxPlan<M>::W, fx_rows_smem<M>(), s>>>(d, ds, ymap);
 }
+template <int M> static void fx_launch_phys(const TcDev& d, int4 zr, cudaStream_t s) {
+    const int pairs = (d.Mz + 1) / 2;
+    kx_phys<M><<<dim3((pairs + FxPlan<M>::G - 1) / FxPlan<M>::G, d.Nr), FxPlan<M>::W, fx_rows_smem<M>() / 5, s>>>(d, zr);
+}
+template <int M> static int4 fx_order() { return make_int4(FxPlan<M>::R0, FxPlan<M>::R1, fx_stride<M, 0>(), fx_stride<M, 1>()); }
 // shared-memory opt-in of the kernels of length M that the axial or the theta
 // transforms use
 template <int M> static void fx_attributes(bool rows, bool z, cudaError_t& e) {
@@ -550,10 +670,12 @@ template <int M> static void fx_attributes(bool rows, bool z, cudaError_t& e) {
     };
     const int zb = fx_z_columns<M>() * (M + M / 8) * (int)sizeof(fxc);
     if (z) { set((const void*)kx_zinv<M>, zb); set((const void*)kx_zfwd<M, false>, zb); set((const void*)kx_zfwd<M, true>, zb); }
-    if (rows) set((const void*)kx_rows<M>, fx_rows_smem<M>());
+    if (rows) { set((const void*)kx_rows<M>, fx_rows_smem<M>()); set((const void*)kx_phys<M>, fx_rows_smem<M>() / 5); }
 }
 #define FX_CASE_Z(M) case M: fx_launch_z<M>(d, ds, ymap, nplanes, which, s, col0, ncols); return true;
 #define FX_CASE_ROWS(M) case M: fx_launch_rows<M>(d, ds, ymap, nplanes, s); return true;
+#define FX_CASE_PHYS(M) case M: fx_launch_phys<M>(d, zr, s); return true;
+#define FX_CASE_ORDER(M) case M: zr = fx_order<M>(); return true;
 #define FX_CASE_ATTR(M) if (Mtx == M || Mzx == M) fx_attributes<M>(Mtx == M, Mzx == M, e);
 // The launchers of one group of lengths: false for a length of another group.
 #define FX_INSTANTIATE(TAG, LIST)                                                                                        \
@@ -564,4 +686,6 @@ template <int M> static void fx_attributes(bool rows, bool z, cudaError_t& e) {
     bool tc_fx_rows_##TAG(const TcDev& d, const TcDev* ds, const int2* ymap, int nplanes, cudaStream_t s) {              \
         switch (d.Mtx) { LIST(FX_CASE_ROWS) default: return false; }                                                    \
     }                                                                                                                   \
+    bool tc_fx_phys_##TAG(const TcDev& d, int4 zr, cudaStream_t s) { switch (d.Mt) { LIST(FX_CASE_PHYS) default: return false; } } \
+    bool tc_fx_order_##TAG(int M, int4& zr) { switch (M) { LIST(FX_CASE_ORDER) default: return false; } }                \
     bool tc_fx_attributes_##TAG(int Mtx, int Mzx, cudaError_t& e) { LIST(FX_CASE_ATTR) return e == cudaSuccess; }

@@ -95,7 +95,7 @@ struct TcDev {
     double* tab_lv;             // [Nr][5][npairs] implicit bands of the v rows and of the eta rows over nu
     double* tab_le;
     double* tab_c;              // [Nr][npairs] c = 1/k^2
-    double* tab_c1;             // [Nr][npairs] c1 = dc/dr
+    double* tab_c1;             // [Nr][npairs] c1 = dc/dr (null in the double-float form, which has tab_c1x)
     float2* tab_cx;             // double-float copies of c, c1 (TC_PREC_DF64 only)
     float2* tab_c1x;
 
@@ -139,13 +139,15 @@ struct TcDev {
     // the quadratic products free of aliasing), tables, and the exponent of
     // 1/(Mtx Mzx), whose mantissa is in the axial table.  fx = 0: Mtx = Mt,
     // Mzx = Mz.
-    int fx, Mtx, Mzx, kexp;
+    // phx: both padded lengths are planned ones themselves, so that the physical
+    // output uses these kernels too (in every form; tables and zexp are then there).
+    int fx, phx, Mtx, Mzx, kexp;
     const fxw* twx_t;
     const fxw* twx_z;
     int* zexp;                  // [3][Nr][Nh]: exponents of zbuf's columns
     int* pexp;                  // [3][Nr][Mzx]: exponents of pbuf's rows (products 0 and 1, 2 and 3, 4)
 
-    // physical output buffer for tc_get_field (float64 [Nr][Mz][Mt])
+    // physical output for tc_get_field (float64 [Nr][Mz][Mt]): pbuf
     double* phys;
     // energy and strain-rate reduction outputs [Nr]
     double* eprof;
@@ -169,6 +171,9 @@ void tc_launch_plane_kernel_batch(const TcDev& d0, const TcDev* ds, const int2* 
 void tc_fx_plane_kernel(const TcDev& d, const TcDev* ds, const int2* ymap, int nplanes, int which, cudaStream_t s,
                         int col0, int ncols);
 cudaError_t tc_fx_attributes(int Mtx, int Mzx);
+// physical output of one field through zbuf, zexp and the tables (phx = 1; false, and
+// nothing launched, otherwise)
+bool tc_fx_to_physical(const TcDev& d, const double2* field, cudaStream_t s);
 cudaError_t tc_probe_fma(double* fp64_tflops, double* fp32_tflops);
 // line phase of all pairs, and of the pairs with azimuthal index j0 <= j < j0 + nj
 // (all axial slots).  mean: with the mean flow (once per substep).  deferred:

@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(128) k_setup(TcDev d) {
     for (int i = 0; i < N; ++i) {
         const Coef q = coef_at(d.r[i], d.rinv[i], m, al);
         d.tab_c[(size_t)i * d.npairs + pair] = q.c;
-        d.tab_c1[(size_t)i * d.npairs + pair] = q.c1;
+        if (d.tab_c1) d.tab_c1[(size_t)i * d.npairs + pair] = q.c1;
         if (d.tab_cx) {
             const dfloat a(q.c), b(q.c1);
             d.tab_cx[(size_t)i * d.npairs + pair] = make_float2(a.hi, a.lo);
@@ -1172,7 +1172,7 @@ __global__ void __launch_bounds__(128) k_init(TcDev d) {
             // band L from the table of k_setup
             for (int s = 0; s < 5; ++s) {
                 const size_t oi = (size_t)(j - 2 + s) * P + pair;
-                const double M5 = d.d0[j * 5 + s] - d.l2[j * 5 + s] * d.tab_c[oi] + d.l1[j * 5 + s] * d.tab_c1[oi];
+                const double M5 = d.d0[j * 5 + s] - d.l2[j * 5 + s] * d.tab_c[oi] + d.l1[j * 5 + s] * (d.tab_c1 ? d.tab_c1[oi] : coef_at(d.r[j - 2 + s], d.rinv[j - 2 + s], m, al).c1);
                 hv = caxpy(hv, M5 + adt * TAB(d.tab_lv, 0, j, s), d.v[oi]);
             }
         }

@@ -19,9 +19,11 @@
 // pair of lengths), and as many radial planes as the array holds go through
 // each pair of launches.
 #include <algorithm>
+#include <array>
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <set>
 #include <string>
 #include <utility>
 #include <vector>
@@ -58,6 +60,14 @@ bool is_smooth(int n) {
     return n == 1;
 }
 
+// radices and strides of a planned length (R0, R1, st0, st1)
+bool fx_order(int M, int4& o) {
+#define FX_ORDER(L) if (M == L) { o = make_int4(FxPlan<L>::R0, FxPlan<L>::R1, fx_stride<L, 0>(), fx_stride<L, 1>()); return true; }
+    FX_LENGTHS(FX_ORDER)
+#undef FX_ORDER
+    return false;
+}
+
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // The z plan (radix 3, 16, then 8/4/2, plus the paired prime stages) and the
@@ -79,9 +89,9 @@ bool plans_for(int Mz, int Mt, FftPlan& pz, FftPlan& pt) {
 }
 
 // Device address of the scratch array for the current device (set-up on the
-// first call per device: symbol address and the shared-memory opt-in of the
+// first call per device and size: symbol address and the shared-memory opt-in of the
 // transform kernels).
-int scratch_for_current_device(unsigned char** out) {
+int scratch_for_current_device(int Mt, int Mz, unsigned char** out) {
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
@@ -102,6 +112,16 @@ int scratch_for_current_device(unsigned char** out) {
             return TC_ERR_CUDA;
         }
         g_scratch_dev[dev] = static_cast<unsigned char*>(p);
+    }
+    // the fixed-point kernels' opt-in, once per device and pair of planned lengths
+    static std::set<std::array<int, 3>> ready;
+    if (ready.find({dev, Mt, Mz}) == ready.end()) {
+        e = tc_fx_attributes(Mt, Mz);
+        if (e != cudaSuccess) {
+            tc_set_error_message(std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
+            return TC_ERR_CUDA;
+        }
+        ready.insert({dev, Mt, Mz});
     }
     *out = g_scratch_dev[dev];
     return TC_OK;
@@ -125,6 +145,52 @@ __global__ void k_noalloc_twiddles(FftPlan p, double2* tw) {
         double sn, cs;
         sincospi(2.0 * (double)num / (double)den, &sn, &cs);
         tw[p.twoff[s] + i] = make_double2(cs, -sn);
+    }
+}
+
+// cos and sin of k/n turns (k < n) times 2^62, to about 2^-61: Taylor series in
+// 64-bit fixed point on the eighth of a turn that k/n falls in (float64 values would
+// add their 2^-53 to every product of the transform).
+__device__ void fx_root(unsigned k, unsigned n, long long& c, long long& s) {
+    typedef unsigned long long u64;
+    const unsigned o = 8 * k / n;
+    unsigned q = 8 * k - o * n;                     // from the eighth's start, or for
+    if (o & 1) q = n - q;                           // odd ones to its end, in 1/(8 n) turns
+    const u64 f = ((u64)q << 32) / n, f1 = (((((u64)q << 32) - f * n) << 31) / n) + (f << 31);   // q/n 2^63
+    const u64 x = __umul64hi(f1, 0xC90FDAA22168C235ull) << 1;                                    // angle 2^64
+    const u64 z = __umul64hi(x, x), one = 1ull << 63;
+    u64 pc = one, ps = one;
+    for (int m = 10; m >= 1; --m) {
+        pc = one - __umul64hi(z, pc) / ((2 * m - 1) * (2 * m));
+        ps = one - __umul64hi(z, ps) / ((2 * m) * (2 * m + 1));
+    }
+    const long long C = (long long)((pc + 1) >> 1);
+    const long long S = (long long)((__umul64hi(x, ps) + 1) >> 1) * (o & 1 ? -1 : 1);
+    switch (((o + 1) >> 1) & 3) {
+        case 0: c = C; s = S; break;
+        case 1: c = -S; s = C; break;
+        case 2: c = -C; s = -S; break;
+        default: c = S; s = -C;
+    }
+}
+
+// Fixed-point twiddles of a planned length (fx_table in tc_fx.cuh without its scaled
+// part): entries [r - 1][tt] of level 0, roots of order M, then of level 1, order n1.
+__global__ void k_noalloc_fx_twiddles(fxw* tw, int M, int st0, int count0, int n1, int st1, int count) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
+        const bool top = i < count0;
+        const int k = top ? i : i - count0, st = top ? st0 : st1, n = top ? M : n1;
+        long long cs, sn;
+        fx_root((unsigned)((k / st + 1) * (k % st)), n, cs, sn);        // (r)(tt) < n
+        auto half = [](long long v, int& h, int& l) {
+            if ((int)v == (int)0x80000000) ++v;                 // the low half can be negated
+            l = (int)v;
+            h = (int)((v - l) >> 32);
+        };
+        fxw w;
+        half(cs, w.rh, w.rl);
+        half(-sn, w.ih, w.il);
+        tw[i] = w;
     }
 }
 
@@ -174,20 +240,43 @@ extern "C" int tc_to_physical_noalloc(int Nr, int Ntheta, int Nz, const void* sp
         return TC_ERR_SIZE;
     }
     unsigned char* scratch = nullptr;
-    int rc = scratch_for_current_device(&scratch);
+    int rc = scratch_for_current_device(d.Mt, d.Mz, &scratch);
     if (rc) return rc;
     cudaStream_t s = (cudaStream_t)cuda_stream;
     // Every call rewrites the twiddles, and the z transform fully writes each
     // plane before the theta transform reads it, so nothing in the array has
     // to start at zero.
-    double2* twz = reinterpret_cast<double2*>(scratch);
-    double2* twt = twz + nz;
-    k_noalloc_twiddles<<<d.pz.nst > 0 ? d.pz.nst : 1, 128, 0, s>>>(d.pz, twz);
-    k_noalloc_twiddles<<<d.pt.nst > 0 ? d.pt.nst : 1, 128, 0, s>>>(d.pt, twt);
-    d.twz_d = twz;
-    d.twt_d = twt;
-    d.zbuf = scratch + tw_bytes;
-    const int chunk = (int)std::min<size_t>((size_t)Nr, ((size_t)TC_NOALLOC_SCRATCH_BYTES - tw_bytes) / plane_bytes);
+    // Both lengths planned: the fixed-point transforms, if their tables and
+    // exponents fit beside a plane.
+    int4 oz, ot;
+    int chunk = 0;
+    if (fx_order(d.Mz, oz) && fx_order(d.Mt, ot)) {
+        auto entries = [](int4 o) { return (o.x - 1) * o.z + (o.w > 1 ? (o.y - 1) * o.w : 0); };
+        const int ez = entries(oz), et = entries(ot);
+        const size_t tab = align256((size_t)(ez + et) * sizeof(fxw)), row = plane_bytes + (size_t)d.Nh * sizeof(int);
+        if (tab + 256 + row <= (size_t)TC_NOALLOC_SCRATCH_BYTES) {
+            fxw* fz = reinterpret_cast<fxw*>(scratch);
+            fxw* ft = fz + ez;
+            k_noalloc_fx_twiddles<<<8, 256, 0, s>>>(fz, d.Mz, oz.z, (oz.x - 1) * oz.z, oz.z, oz.w, ez);
+            k_noalloc_fx_twiddles<<<8, 256, 0, s>>>(ft, d.Mt, ot.z, (ot.x - 1) * ot.z, ot.z, ot.w, et);
+            chunk = (int)std::min<size_t>((size_t)Nr, ((size_t)TC_NOALLOC_SCRATCH_BYTES - tab - 256) / row);
+            d.phx = 1;
+            d.twx_z = fz;
+            d.twx_t = ft;
+            d.zexp = reinterpret_cast<int*>(scratch + tab);
+            d.zbuf = scratch + tab + align256((size_t)chunk * d.Nh * sizeof(int));
+        }
+    }
+    if (!d.phx) {
+        double2* twz = reinterpret_cast<double2*>(scratch);
+        double2* twt = twz + nz;
+        k_noalloc_twiddles<<<d.pz.nst > 0 ? d.pz.nst : 1, 128, 0, s>>>(d.pz, twz);
+        k_noalloc_twiddles<<<d.pt.nst > 0 ? d.pt.nst : 1, 128, 0, s>>>(d.pt, twt);
+        d.twz_d = twz;
+        d.twt_d = twt;
+        d.zbuf = scratch + tw_bytes;
+        chunk = (int)std::min<size_t>((size_t)Nr, ((size_t)TC_NOALLOC_SCRATCH_BYTES - tw_bytes) / plane_bytes);
+    }
     const double2* spec = static_cast<const double2*>(spectral_dev);
     double* phys = static_cast<double*>(physical_dev);
     for (int r0 = 0; r0 < Nr; r0 += chunk) {

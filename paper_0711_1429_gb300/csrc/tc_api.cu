@@ -1433,14 +1433,12 @@ int tc_torque_stats(tc_handle* h, tc_stats* out) {
     if ((rc = ensure_init(h))) return rc;
     TcDev& d = h->d;
     const int N = d.Nr;
-    std::vector<double> W(N), ep(N), dp(N);
-    tc_launch_energy(d, h->stream);
-    tc_launch_strain(d, h->stream);
+    std::vector<double> prof(5 * (size_t)N);     // W, HU, HW, eprof, dprof as they lie on the device
+    tc_launch_diagnostics(d, h->stream);
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(W.data(), d.W, N * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaMemcpyAsync(ep.data(), d.eprof, N * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaMemcpyAsync(dp.data(), d.dprof, N * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaMemcpyAsync(prof.data(), d.W, 5 * (size_t)N * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
+    const double *W = prof.data(), *ep = W + 3 * N, *dp = W + 4 * N;
     const double* e0 = &h->S.dwall[0];
     const double* e1 = &h->S.dwall[5];
     double dWi = 0, dWo = 0;

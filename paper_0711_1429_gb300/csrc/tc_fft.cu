@@ -1,6 +1,6 @@
 // Plane phase: dispatch to the per-type kernels (tc_fft_f64.cu, tc_fft_f32.cu,
 // tc_fft_df.cu; templates and the description of the transforms in
-// tc_fft_impl.cuh), the transform-length table and the energy reduction.
+// tc_fft_impl.cuh; fixed point: tc_fx_*.cu) and the transform-length table.
 #include "tc_internal.h"
 
 void tc_plane_kernel_f64(const TcDev& d, int which, cudaStream_t s, int tile0, int ntiles);
@@ -61,27 +61,6 @@ bool tc_fft_fixed_length(int M) {
     return false;
 }
 
-// ---- kinetic-energy profile: sum over pairs of weight |u|^2+|v|^2+|w|^2 ------
-__global__ void __launch_bounds__(256) k_energy(TcDev d) {
-    const int r = blockIdx.x;
-    double acc = 0.0;
-    for (int i = threadIdx.x; i < d.npairs; i += blockDim.x) {
-        const int j = i % d.Nh;
-        const size_t o = (size_t)r * d.npairs + i;
-        const double2 a = d.u[o], b = d.v[o], c = d.w[o];
-        const double wgt = j == 0 ? 1.0 : 2.0;
-        acc += wgt * (a.x * a.x + a.y * a.y + b.x * b.x + b.y * b.y + c.x * c.x + c.y * c.y);
-    }
-    __shared__ double red[256];
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) d.eprof[r] = red[0];
-}
-
 void tc_launch_plane_kernel_tiles(const TcDev& d, int which, cudaStream_t s, int tile0, int ntiles) {
     if (d.fx) tc_fx_plane_kernel(d, nullptr, nullptr, d.Nr, which, s, tile0 * d.ztile, ntiles * d.ztile);
     else if (d.prec == 1) tc_plane_kernel_f32(d, which, s, tile0, ntiles);
@@ -113,8 +92,4 @@ cudaError_t tc_set_kernel_attributes() {
                           tc_rows_phys_attributes()})
         if (r != cudaSuccess) e = r;
     return e;
-}
-
-void tc_launch_energy(const TcDev& d, cudaStream_t s) {
-    k_energy<<<d.Nr, 256, 0, s>>>(d);
 }

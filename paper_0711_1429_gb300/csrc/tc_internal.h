@@ -202,11 +202,10 @@ void tc_launch_init_state(const TcDev& d, cudaStream_t s);
 // zero the (0,0) and Nyquist slots and make the m = 0 column Hermitian
 void tc_launch_realify(const TcDev& d, double2* field, cudaStream_t s);
 void tc_launch_to_physical(const TcDev& d, const double2* field, cudaStream_t s);
-void tc_launch_energy(const TcDev& d, cudaStream_t s);
 // transform lengths with a compile-time plan in the FFT kernels
 bool tc_fft_fixed_length(int M);
-// sum over Fourier slots of 2 S:S at every radial point -> d.dprof
-// (scratch: pbuf for the radial derivatives, zbuf for the densities)
-void tc_launch_strain(const TcDev& d, cudaStream_t s);
+// sums over the Fourier slots of |u|^2 and 2 S:S at every radial point -> d.eprof,
+// d.dprof (scratch: pbuf for the radial derivatives, zbuf for the densities)
+void tc_launch_diagnostics(const TcDev& d, cudaStream_t s);
 cudaError_t tc_set_kernel_attributes();
 cudaError_t tc_set_line_kernel_attributes();

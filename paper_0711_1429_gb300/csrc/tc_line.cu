@@ -286,96 +286,6 @@ __global__ void __launch_bounds__(128) k_setup(TcDev d) {
 }
 
 // ---------------------------------------------------------------------------
-// u, w from v, eta (continuity and the definition of eta):
-//   Dv: 0 on rows 0, Nr-1; explicit one-sided rows 1, Nr-2; compact rows
-//       d0 . Dv = l1 . v on rows 2..Nr-3 (solved with the reversed
-//       factorisation dsol, the elimination running from the outer wall in);
-//   u = (i alpha D_*v - (i m/r) eta)/k^2,   w = ((i m/r) D_*v + i alpha eta)/k^2.
-// z_j of the elimination is kept in u[j] until the ascending pass.
-__device__ void reconstruct_pair(const TcDev& d, int pair, double m, double al, long long partner) {
-    const int N = d.Nr;
-    const size_t P = d.npairs;
-    double2 xw[5];
-    for (int s = 0; s < 5; ++s) xw[s] = cz();
-    double2 Dv1 = cz(), DvN = cz();
-    double2 z1 = cz(), z2 = cz();     // z_{jr+1}, z_{jr+2}
-    double2 r3 = cz(), r2 = cz();
-    auto known = [&](int jr, double2 rhs) -> double2 {
-        const double* w0 = d.d0 + jr * 5;
-        if (jr + 1 == N - 2) rhs = caxpy(rhs, -w0[3], DvN);
-        if (jr + 2 == N - 2) rhs = caxpy(rhs, -w0[4], DvN);
-        if (jr - 1 == 1) rhs = caxpy(rhs, -w0[1], Dv1);
-        if (jr - 2 == 1) rhs = caxpy(rhs, -w0[0], Dv1);
-        return rhs;
-    };
-    auto elim = [&](int jr, double2 rhs) {
-        const double* q = d.dsol + jr * 5;
-        double2 z = caxpy(caxpy(known(jr, rhs), -q[0], z2), -q[1], z1);
-        d.u[(size_t)jr * P + pair] = z;
-        z2 = z1;
-        z1 = z;
-    };
-    for (int i = N - 1; i >= 0; --i) {
-        for (int s = 4; s > 0; --s) xw[s] = xw[s - 1];
-        xw[0] = d.v[(size_t)i * P + pair];
-        if (i > N - 5) continue;
-        if (i == N - 5) {                       // one-sided row N-2
-            const double* w = d.l1 + (N - 2) * 5;
-            double2 acc = cz();
-            for (int s = 0; s < 5; ++s) acc = caxpy(acc, w[s], xw[s]);
-            DvN = acc;
-        }
-        const int jr = i + 2;
-        if (jr >= 2 && jr <= N - 3) {
-            const double* w = d.l1 + jr * 5;
-            double2 acc = cz();
-            for (int s = 0; s < 5; ++s) acc = caxpy(acc, w[s], xw[s]);
-            if (jr >= 4) elim(jr, acc);
-            else if (jr == 3) r3 = acc;
-            else r2 = acc;
-        }
-        if (i == 0) {                           // one-sided row 1
-            const double* w = d.l1 + 1 * 5;
-            double2 acc = cz();
-            for (int s = 0; s < 5; ++s) acc = caxpy(acc, w[s], xw[s]);
-            Dv1 = acc;
-        }
-    }
-    if (N - 3 >= 3) elim(3, r3);
-    elim(2, r2);
-    // ascending: back substitution and u, w
-    double2 p1 = cz(), p2 = cz();               // Dv_{i-1}, Dv_{i-2} among unknowns 2..N-3
-    for (int i = 0; i < N; ++i) {
-        double2 Dv;
-        if (i == 0 || i == N - 1) Dv = cz();
-        else if (i == 1) Dv = Dv1;
-        else if (i == N - 2) Dv = DvN;
-        else {
-            const double* q = d.dsol + i * 5;
-            const double2 z = d.u[(size_t)i * P + pair];
-            Dv = cscale(q[2], caxpy(caxpy(z, -q[3], p1), -q[4], p2));
-            p2 = p1;
-            p1 = Dv;
-        }
-        const double ri = d.rinv[i];
-        const double c = d.tab_c[(size_t)i * P + pair];
-        const double2 V = d.v[(size_t)i * P + pair];
-        const double2 E = d.eta[(size_t)i * P + pair];
-        const double2 Dsv = caxpy(Dv, ri, V);
-        // u = i (c alpha Dsv - c m/r eta), w = i (c m/r Dsv + c alpha eta)
-        const double ca = c * al, cm = c * m * ri;
-        const double2 uu = ci(make_double2(fma(ca, Dsv.x, -cm * E.x), fma(ca, Dsv.y, -cm * E.y)));
-        const double2 ww = ci(make_double2(fma(cm, Dsv.x, ca * E.x), fma(cm, Dsv.y, ca * E.y)));
-        d.u[(size_t)i * P + pair] = uu;
-        d.w[(size_t)i * P + pair] = ww;
-        if (partner >= 0) {
-            d.u[(size_t)i * P + partner] = cconj(uu);
-            d.w[(size_t)i * P + partner] = cconj(ww);
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
 // The line phase of one substep, for the pairs of the azimuthal columns
 // ja .. ja + jw - 1 in every axial slot (all pairs when ja = 0, jw = Ntheta/2):
 // two kernels.
@@ -507,8 +417,12 @@ __device__ __forceinline__ void rk_memory_row(const TcDev& d, const double* __re
     H[2 * (size_t)jr * d.npairs] = fma(hdt, acc, H[2 * (size_t)jr * d.npairs]);
 }
 // The rows centred on i0 <= i < i1 (v: 2 .. Nr - 3; the one-sided eta rows 1 and
-// Nr - 2 with their neighbours).
-__device__ __forceinline__ void rk_memory_rows(const TcDev& d, int k, int pair, int comp, int i0, int i1) {
+// Nr - 2 with their neighbours).  BAND: the eta band is formed here instead of read,
+// with the table's own operations, where the float64 pipe has time to spare but not
+// the memory: beside the mixed form's theta rows.
+template <bool BAND = false>
+__device__ __forceinline__ void rk_memory_rows(const TcDev& d, int k, int pair, int comp, int i0, int i1, double m = 0.0,
+                                               double al = 0.0) {
     const int N = d.Nr, kn = (k + 1) % 3;
     const size_t P2 = 2 * (size_t)d.npairs;
     const double hdt = (d.rk_beta[k] + d.rk_alpha[kn]) * d.dt, hdtnu = hdt * d.nu;
@@ -520,14 +434,30 @@ __device__ __forceinline__ void rk_memory_rows(const TcDev& d, int k, int pair, 
     if (i0 >= i1) return;
     double xv[5], xe[5];
     for (int s = 0; s < 4; ++s) { xv[s + 1] = v[(i0 - 2 + s) * P2]; xe[s + 1] = e[(i0 - 2 + s) * P2]; }
+    double k2[5];
+    if constexpr (BAND)
+        for (int s = 0; s < 4; ++s) k2[s + 1] = k2_at(m, al, d.rinv[i0 - 2 + s]);
+    auto eta_row = [&](int j) {
+        if constexpr (BAND) {
+            double acc = 0.0;
+            for (int s = 0; s < 5; ++s) acc = fma(fma(-d.d0[j * 5 + s], k2[s], d.l2[j * 5 + s]), xe[s], acc);
+            He[(size_t)j * P2] = fma(hdtnu, acc, He[(size_t)j * P2]);
+        } else {
+            rk_memory_row(d, d.tab_le, He, pair, j, xe, hdtnu);
+        }
+    };
     for (int i = i0; i < i1; ++i) {
         for (int s = 0; s < 4; ++s) { xv[s] = xv[s + 1]; xe[s] = xe[s + 1]; }
+        if constexpr (BAND) {
+            for (int s = 0; s < 4; ++s) k2[s] = k2[s + 1];
+            k2[4] = k2_at(m, al, d.rinv[i + 2]);
+        }
         xv[4] = v[(i + 2) * P2];
         xe[4] = e[(i + 2) * P2];
         rk_memory_row(d, d.tab_lv, Hv, pair, i, xv, hdt);
-        rk_memory_row(d, d.tab_le, He, pair, i, xe, hdtnu);
-        if (i == 2) rk_memory_row(d, d.tab_le, He, pair, 1, xe, hdtnu);
-        if (i == N - 3) rk_memory_row(d, d.tab_le, He, pair, N - 2, xe, hdtnu);
+        eta_row(i);
+        if (i == 2) eta_row(1);
+        if (i == N - 3) eta_row(N - 2);
     }
 }
 
@@ -1149,46 +1079,59 @@ __global__ void __launch_bounds__(128) k_rk_memory(TcDev d, int k, int ja, int j
         int pair;
         double m, al;
         long long partner;
-        if (line_pair(d, ja, jw, idx >> 1, pair, m, al, partner)) rk_memory_rows(d, k, pair, idx & 1, 0, d.Nr);
+        if (line_pair(d, ja, jw, idx >> 1, pair, m, al, partner)) rk_memory_rows<true>(d, k, pair, idx & 1, 0, d.Nr, m, al);
     }
 }
 
 // ---------------------------------------------------------------------------
-// Initial RK memory H_1 = (M + alpha_1 dt L) x for v and eta, and u, w.
-__global__ void __launch_bounds__(128) k_init(TcDev d) {
-    const int pair = blockIdx.x * blockDim.x + threadIdx.x;
-    if (pair >= d.npairs) return;
-    double m, al;
-    long long partner;
-    if (!pair_info(d, pair, m, al, partner)) return;
+// Initial RK memory H_1 = (M + alpha_1 dt L) x for v and eta, and u, w, as k_solve
+// after its solves: the rows i0 <= i < i1 of H_1.
+__device__ __forceinline__ void init_rows(const TcDev& d, int pair, int comp, double m, double al, int i0, int i1) {
     const int N = d.Nr;
-    const size_t P = d.npairs;
+    const size_t P = d.npairs, P2 = 2 * P, o = 2 * (size_t)pair + comp;
     const double adt = d.rk_alpha[0] * d.dt;
-    for (int j = 0; j < N; ++j) {
-        const size_t o = (size_t)j * P + pair;
-        double2 hv = cz(), he = cz();
+    const double *v = reinterpret_cast<const double*>(d.v) + o, *e = reinterpret_cast<const double*>(d.eta) + o;
+    double *Hv = reinterpret_cast<double*>(d.Hv) + o, *He = reinterpret_cast<double*>(d.He) + o;
+    for (int j = i0; j < i1; ++j) {
+        double hv = 0.0, he = 0.0;
         if (j >= 2 && j <= N - 3) {
-            // mass band M = d0 - l2 c + l1 c' from the c, c' tables, implicit
-            // band L from the table of k_setup
+            // mass band M = d0 - l2 c + l1 c' from the c, c' tables
             for (int s = 0; s < 5; ++s) {
-                const size_t oi = (size_t)(j - 2 + s) * P + pair;
-                const double M5 = d.d0[j * 5 + s] - d.l2[j * 5 + s] * d.tab_c[oi] + d.l1[j * 5 + s] * (d.tab_c1 ? d.tab_c1[oi] : coef_at(d.r[j - 2 + s], d.rinv[j - 2 + s], m, al).c1);
-                hv = caxpy(hv, M5 + adt * TAB(d.tab_lv, 0, j, s), d.v[oi]);
+                const size_t i = j - 2 + s;
+                const double M5 = d.d0[j * 5 + s] - d.l2[j * 5 + s] * d.tab_c[i * P + pair] + d.l1[j * 5 + s] * (d.tab_c1 ? d.tab_c1[i * P + pair] : coef_at(d.r[i], d.rinv[i], m, al).c1);
+                hv = fma(M5 + adt * TAB(d.tab_lv, 0, j, s), v[i * P2], hv);
             }
         }
         if (j >= 1 && j <= N - 2) {
-            const int st = d.start[j];
+            const size_t st = d.start[j];
             for (int s = 0; s < 5; ++s) {
                 const double ri = d.rinv[st + s];
                 const double L5 = d.nu * (d.l2[j * 5 + s] - d.d0[j * 5 + s] * (al * al + m * m * ri * ri));
-                const double2 x = d.eta[(size_t)(st + s) * P + pair];
-                he = caxpy(he, d.d0[j * 5 + s] + adt * L5, x);
+                he = fma(d.d0[j * 5 + s] + adt * L5, e[(st + s) * P2], he);
             }
         }
-        d.Hv[o] = hv;
-        d.He[o] = he;
+        Hv[(size_t)j * P2] = hv;
+        He[(size_t)j * P2] = he;
     }
-    reconstruct_pair(d, pair, m, al, partner);
+}
+template <int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, WARPS > 2 ? 2 : 12) k_init(const __grid_constant__ TcDev d) {
+    const int warp = threadIdx.x >> 5, comp = threadIdx.x & 1;
+    int pair = 0;
+    double m = 0.0, al = 0.0;
+    long long partner = -1;
+    const bool act = line_pair(d, 0, d.Nh, blockIdx.x * 16 + ((threadIdx.x & 31) >> 1), pair, m, al, partner);
+    const RowTables t{d.d0, d.l1, d.dsol, d.rinv};
+    double* S = reinterpret_cast<double*>(rhs_scratch(d, pair)) + comp;
+    const int N = d.Nr;
+    if (act) derivative_rows(d, t, reinterpret_cast<const double*>(d.v) + 2 * (size_t)pair + comp, S, warp * N / WARPS, (warp + 1) * N / WARPS);
+    __syncthreads();
+    if (act) {
+        if (warp == 0) derivative_solve(d, t, S);
+        else init_rows(d, pair, comp, m, al, (warp - 1) * N / (WARPS - 1), warp * N / (WARPS - 1));
+    }
+    __syncthreads();
+    if (act) velocity_rows(d, t, pair, comp, m, al, partner, S, warp * N / WARPS, (warp + 1) * N / WARPS);
 }
 
 // ---------------------------------------------------------------------------
@@ -1481,112 +1424,124 @@ k_explicit_b(const TcDev* __restrict__ ds, const int2* __restrict__ emap, int k,
 }
 
 // ---------------------------------------------------------------------------
-// Diagnostics: strain-rate density for the viscous dissipation.
+// Diagnostics: kinetic energy and strain-rate density, every Fourier slot (the (0,0)
+// slot holds the mean flow U, W), 16 slots a block, a lane per component as in
+// k_solve.  (One thread per slot was the latency of six recurrences and an energy kernel
+// that read u, v, w again: a restart of 129x128x128 with its statistics, k_init with a
+// thread per pair included, 1662 -> 670 us.)
 //
-// compact_D: first radial derivative of one Fourier slot of a field, the
-// operator of the energy budget: explicit one-sided 5-point D on the walls
-// (dwall) and on rows 1, Nr-2 (l1 rows with d0 = 1), compact rows
-// d0 . Df = l1 . f on 2..Nr-3 solved with the reversed factorisation dsol
-// (descending elimination, z kept in Df, then ascending substitution).
-__device__ void compact_D(const TcDev& d, const double2* __restrict__ f, double2* Df, int pair) {
-    const int N = d.Nr;
-    const size_t P = d.npairs;
-    auto F = [&](int i) { return f[(size_t)i * P + pair]; };
-    double2 D0 = cz(), D1 = cz(), DN2 = cz(), DN1 = cz();
-    for (int s = 0; s < 5; ++s) {
-        D0 = caxpy(D0, d.dwall[s], F(s));
-        DN1 = caxpy(DN1, d.dwall[5 + s], F(N - 5 + s));
-        D1 = caxpy(D1, d.l1[5 + s], F(d.start[1] + s));
-        DN2 = caxpy(DN2, d.l1[(N - 2) * 5 + s], F(d.start[N - 2] + s));
-    }
-    double2 z1 = cz(), z2 = cz();               // z_(jr+1), z_(jr+2)
-    for (int jr = N - 3; jr >= 2; --jr) {
-        const double* w0 = d.d0 + jr * 5;
-        const double* w1 = d.l1 + jr * 5;
-        double2 rhs = cz();
-        for (int s = 0; s < 5; ++s) {
-            const int c = jr - 2 + s;
-            rhs = caxpy(rhs, w1[s], F(c));
-            if (c == 0) rhs = caxpy(rhs, -w0[s], D0);
-            else if (c == 1) rhs = caxpy(rhs, -w0[s], D1);
-            else if (c == N - 2) rhs = caxpy(rhs, -w0[s], DN2);
-            else if (c == N - 1) rhs = caxpy(rhs, -w0[s], DN1);
-        }
-        const double* q = d.dsol + jr * 5;
-        const double2 z = caxpy(caxpy(rhs, -q[0], z2), -q[1], z1);
-        Df[(size_t)jr * P + pair] = z;
-        z2 = z1;
-        z1 = z;
-    }
-    double2 p1 = cz(), p2 = cz();               // Df_(i-1), Df_(i-2) among 2..Nr-3
-    for (int i = 2; i <= N - 3; ++i) {
-        const double* q = d.dsol + i * 5;
-        const double2 x = cscale(q[2], caxpy(caxpy(Df[(size_t)i * P + pair], -q[3], p1), -q[4], p2));
-        Df[(size_t)i * P + pair] = x;
-        p2 = p1;
-        p1 = x;
-    }
-    Df[pair] = D0;
-    Df[P + pair] = D1;
-    Df[(size_t)(N - 2) * P + pair] = DN2;
-    Df[(size_t)(N - 1) * P + pair] = DN1;
-}
-
-__device__ __forceinline__ double cabs2(double2 a) { return a.x * a.x + a.y * a.y; }
-
-// One thread per Fourier slot (every slot; the (0,0) slot holds the mean
-// flow U, W): 2 S:S with the cylindrical strain components
+// First radial derivative of u, v and w, the operator of the energy budget: explicit
+// one-sided 5-point D on the walls (dwall) and on rows 1, Nr-2 (l1 rows with d0 = 1),
+// compact rows d0 . Df = l1 . f on 2..Nr-3 solved with the reversed factorisation
+// dsol.  All warps share the right sides by rows, one warp per field runs its
+// recurrences, then all share the densities: 2 S:S with the cylindrical strain
+// components
 //   S_rr = Dv, S_tt = (i m/r) w + v/r, S_zz = i alpha u,
 //   S_rt = (Dw - w/r + (i m/r) v)/2, S_rz = (i alpha v + Du)/2,
 //   S_tz = ((i m/r) u + i alpha w)/2,
-// times the Parseval weight (1 for m = 0, 2 otherwise), into dens[r][slot].
-__global__ void __launch_bounds__(128) k_strain(TcDev d, double2* Du, double2* Dv, double2* Dw, double* dens) {
-    const int pair = blockIdx.x * blockDim.x + threadIdx.x;
-    if (pair >= d.npairs) return;
-    const int sl = pair / d.Nh, j = pair - sl * d.Nh;
+// and |u|^2 + |v|^2 + |w|^2, times the Parseval weight (1 for m = 0, 2 otherwise), into
+// dens[0] and dens[1], [r][slot].
+constexpr int DIAG_WARPS = 4;
+__global__ void __launch_bounds__(32 * DIAG_WARPS)
+k_strain(const __grid_constant__ TcDev d, double* __restrict__ D, double* __restrict__ dens) {
+    const int warp = threadIdx.x >> 5, comp = threadIdx.x & 1;
+    const int pair = blockIdx.x * 16 + ((threadIdx.x & 31) >> 1);
+    const bool act = pair < d.npairs;
+    const int N = d.Nr;
+    const size_t P = d.npairs, P2 = 2 * P, o = act ? 2 * (size_t)pair + comp : comp;
+    const double* f[3] = {reinterpret_cast<const double*>(d.u), reinterpret_cast<const double*>(d.v), reinterpret_cast<const double*>(d.w)};
+    const int i0 = warp * N / DIAG_WARPS, i1 = (warp + 1) * N / DIAG_WARPS;
+    if (act) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const double* F = f[q] + o;
+            double* R = D + q * N * P2 + o;
+            for (int j = i0; j < i1; ++j) {
+                const int st = j < 2 ? 0 : j > N - 3 ? N - 5 : j - 2;
+                const double* w = j == 0 ? d.dwall : j == N - 1 ? d.dwall + 5 : d.l1 + j * 5;
+                double acc = 0.0;
+                for (int s = 0; s < 5; ++s) acc = fma(w[s], F[(size_t)(st + s) * P2], acc);
+                R[(size_t)j * P2] = acc;
+            }
+        }
+    }
+    __syncthreads();
+    if (act && warp < 3) {
+        double* R = D + warp * N * P2 + o;
+        const double D0 = R[0], D1 = R[P2], DM = R[(size_t)(N - 2) * P2], DN = R[(size_t)(N - 1) * P2];
+        double z1 = 0.0, z2 = 0.0;
+        rows_ahead<OneRow>(
+            N - 4, [&](int q, OneRow& w) { w.z = R[(size_t)(N - 3 - q) * P2]; },
+            [&](int q, const OneRow& w) {
+                const int j = N - 3 - q;
+                const double* w0 = d.d0 + j * 5;
+                double r = w.z;
+                if (j == 2) r = fma(-w0[1], D1, fma(-w0[0], D0, r));
+                if (j == 3) r = fma(-w0[0], D1, r);
+                if (j == N - 4) r = fma(-w0[4], DM, r);
+                if (j == N - 3) r = fma(-w0[4], DN, fma(-w0[3], DM, r));
+                const double* c = d.dsol + j * 5;
+                const double z = fma(-c[1], z1, fma(-c[0], z2, r));
+                R[(size_t)j * P2] = z;
+                z2 = z1; z1 = z;
+            });
+        double p1 = 0.0, p2 = 0.0;
+        rows_ahead<OneRow>(
+            N - 4, [&](int q, OneRow& w) { w.z = R[(size_t)(q + 2) * P2]; },
+            [&](int q, const OneRow& w) {
+                const double* c = d.dsol + (q + 2) * 5;
+                const double x = c[2] * fma(-c[4], p2, fma(-c[3], p1, w.z));
+                R[(size_t)(q + 2) * P2] = x;
+                p2 = p1; p1 = x;
+            });
+    }
+    __syncthreads();
+    const int sl = act ? pair / d.Nh : 0, j = act ? pair - sl * d.Nh : 0;
     const int n = sl < d.Nz / 2 ? sl : (sl == d.Nz / 2 ? 0 : sl - d.Nz);
     const double m = j * d.m0, al = n * d.alpha0;
-    const double wgt = j == 0 ? 1.0 : 2.0;
-    compact_D(d, d.u, Du, pair);
-    compact_D(d, d.v, Dv, pair);
-    compact_D(d, d.w, Dw, pair);
-    const size_t P = d.npairs;
-    for (int i = 0; i < d.Nr; ++i) {
-        const size_t o = (size_t)i * P + pair;
-        const double ri = d.rinv[i];
-        const double2 U = d.u[o], V = d.v[o], W = d.w[o];
-        const double2 srr = Dv[o];
-        const double2 stt = caxpy(cimag(m * ri, W), ri, V);
-        const double2 szz = cimag(al, U);
-        const double2 srt = cscale(0.5, cadd(caxpy(Dw[o], -ri, W), cimag(m * ri, V)));
-        const double2 srz = cscale(0.5, cadd(cimag(al, V), Du[o]));
-        const double2 stz = cscale(0.5, cadd(cimag(m * ri, U), cimag(al, W)));
-        dens[o] = wgt * (2.0 * (cabs2(srr) + cabs2(stt) + cabs2(szz)) +
-                         4.0 * (cabs2(srt) + cabs2(srz) + cabs2(stz)));
+    const double wgt = j == 0 ? 1.0 : 2.0, sg = comp ? 1.0 : -1.0;      // i a: other component times sg
+    const double *Du = D + o, *Dv = D + N * P2 + o, *Dw = D + 2 * N * P2 + o;
+    const size_t x = o + 1 - 2 * comp;
+    for (int i = i0; i < i1; ++i) {
+        const size_t row = (size_t)i * P2;
+        const double ri = d.rinv[i], imr = sg * m * ri, ial = sg * al;
+        const double U = f[0][o + row], V = f[1][o + row], W = f[2][o + row];
+        const double Ux = f[0][x + row], Vx = f[1][x + row], Wx = f[2][x + row];
+        const double srr = Dv[row], stt = fma(imr, Wx, ri * V), szz = ial * Ux;
+        const double srt = fma(imr, Vx, fma(-ri, W, Dw[row])), srz = fma(ial, Vx, Du[row]), stz = fma(imr, Ux, ial * Wx);
+        double a = wgt * fma(2.0, fma(srr, srr, fma(stt, stt, szz * szz)), fma(srt, srt, fma(srz, srz, stz * stz)));
+        double b = wgt * fma(U, U, fma(V, V, W * W));
+        a += __shfl_xor_sync(0xffffffffu, a, 1);
+        b += __shfl_xor_sync(0xffffffffu, b, 1);
+        if (act) dens[(size_t)comp * N * P + (size_t)i * P + pair] = comp ? b : a;
     }
 }
 
-// dprof[r] = sum over slots of dens[r][slot] (fixed order: reproducible)
+// dprof[r], eprof[r] = sums over the slots of dens[0][r], dens[1][r] (fixed order:
+// reproducible)
 __global__ void __launch_bounds__(256) k_slot_sum(TcDev d, const double* __restrict__ dens) {
     const int r = blockIdx.x;
-    double acc = 0.0;
-    for (int i = threadIdx.x; i < d.npairs; i += blockDim.x) acc += dens[(size_t)r * d.npairs + i];
+    const double* x = dens + ((size_t)blockIdx.y * d.Nr + r) * d.npairs;
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int i = threadIdx.x; i < d.npairs; i += 4 * blockDim.x)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (i + q * (int)blockDim.x < d.npairs) a[q] += x[i + q * blockDim.x];
     __shared__ double red[256];
-    red[threadIdx.x] = acc;
+    red[threadIdx.x] = (a[0] + a[1]) + (a[2] + a[3]);
     __syncthreads();
     for (int s = blockDim.x / 2; s > 0; s >>= 1) {
         if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
         __syncthreads();
     }
-    if (threadIdx.x == 0) d.dprof[r] = red[0];
+    if (threadIdx.x == 0) (blockIdx.y ? d.eprof : d.dprof)[r] = red[0];
 }
 
-void tc_launch_strain(const TcDev& d, cudaStream_t s) {
-    const size_t P1 = (size_t)d.Nr * d.npairs;   // <= Nr Mz Nh: fits the scratch
-    double2* D = reinterpret_cast<double2*>(d.pbuf);
+void tc_launch_diagnostics(const TcDev& d, cudaStream_t s) {
+    double* D = reinterpret_cast<double*>(d.pbuf);      // 3 Nr npairs complex, of TC_NPROD Nr Mzx Nh
     double* dens = reinterpret_cast<double*>(d.zbuf);
-    k_strain<<<(d.npairs + 127) / 128, 128, 0, s>>>(d, D, D + P1, D + 2 * P1, dens);
-    k_slot_sum<<<d.Nr, 256, 0, s>>>(d, dens);
+    k_strain<<<(d.npairs + 15) / 16, 32 * DIAG_WARPS, 0, s>>>(d, D, dens);
+    k_slot_sum<<<dim3(d.Nr, 2), 256, 0, s>>>(d, dens);
 }
 
 // ---------------------------------------------------------------------------
@@ -1763,6 +1718,8 @@ cudaError_t tc_set_line_kernel_attributes() {
 }
 
 void tc_launch_init_state(const TcDev& d, cudaStream_t s) {
-    k_init<<<(d.npairs + 127) / 128, 128, 0, s>>>(d);
+    const int half = (d.npairs + 15) / 16;
+    if (half < WIDE_GROUPS) k_init<8><<<half, 256, 0, s>>>(d);
+    else k_init<2><<<half, 64, 0, s>>>(d);
     k_mean_init<<<1, 256, 0, s>>>(d);
 }

@@ -44,12 +44,6 @@ __device__ __forceinline__ Coef coef_at(double r, double rinv, double m, double 
 }
 
 __device__ __forceinline__ double2 cz() { return make_double2(0.0, 0.0); }
-__device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ double2 cscale(double s, double2 a) { return make_double2(s * a.x, s * a.y); }
-// (i s) * a
-__device__ __forceinline__ double2 cimag(double s, double2 a) { return make_double2(-s * a.y, s * a.x); }
-// i * a
-__device__ __forceinline__ double2 ci(double2 a) { return make_double2(-a.y, a.x); }
 // a + s * b
 __device__ __forceinline__ double2 caxpy(double2 a, double s, double2 b) { return make_double2(fma(s, b.x, a.x), fma(s, b.y, a.y)); }
 __device__ __forceinline__ double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
@@ -61,7 +55,6 @@ __device__ __forceinline__ double2 ld_prod(const float2* p, size_t o) { float2 f
 
 // generic complex helpers for float2 / double2
 template <typename CT> __device__ __forceinline__ CT tz() { CT r; r.x = 0; r.y = 0; return r; }
-template <typename CT, typename T> __device__ __forceinline__ CT timag(T s, CT a) { CT r; r.x = -s * a.y; r.y = s * a.x; return r; }
 template <typename CT> __device__ __forceinline__ CT tadd(CT a, CT b) { CT r; r.x = a.x + b.x; r.y = a.y + b.y; return r; }
 template <typename CT> __device__ __forceinline__ CT tsub(CT a, CT b) { CT r; r.x = a.x - b.x; r.y = a.y - b.y; return r; }
 template <typename CT, typename T> __device__ __forceinline__ CT taxpy(CT a, T s, CT b) { CT r; r.x = fma(s, b.x, a.x); r.y = fma(s, b.y, a.y); return r; }
@@ -488,7 +481,7 @@ __device__ __forceinline__ double2* rhs_scratch(const TcDev& d, int pair) {
 constexpr int EXPLICIT_WARPS = 4;
 template <int MODE> struct RowRing {
     typedef typename LineTypes<MODE>::CT CT;
-    static constexpr int RING = MODE == 1 ? 4 : MODE == 2 ? 3 : 0, NT = 32 * EXPLICIT_WARPS;
+    static constexpr int RING = MODE > 0 ? 3 : 0, NT = 32 * EXPLICIT_WARPS;
     static constexpr int FIELDS = 5 * sizeof(CT) * NT, H = FIELDS + 48 * NT, COEF = H + 32 * NT, BYTES = COEF + 16 * NT;
     unsigned char* base;
     __device__ CT& prod(int q) const { return *reinterpret_cast<CT*>(base + (q * NT + threadIdx.x) * sizeof(CT)); }
@@ -1303,7 +1296,7 @@ __device__ __forceinline__ void explicit_body(const TcDev& d, int k, int ja, int
     explicit_rows<MODE>(d, k, ja, jw, pg * 32 + (threadIdx.x & 31), c0, c1);
 }
 template <int MODE>
-__global__ void __launch_bounds__(32 * EXPLICIT_WARPS, 3)
+__global__ void __launch_bounds__(32 * EXPLICIT_WARPS, MODE == 1 ? 4 : 3)
 k_explicit(const __grid_constant__ TcDev d, int k, int ja, int jw, int Lc, int mean) {
     if (mean && blockIdx.x == gridDim.x - 1) mean_body<typename LineTypes<MODE>::CT>(d, k);
     else explicit_body<MODE>(d, k, ja, jw, Lc, blockIdx.x);
@@ -1415,7 +1408,7 @@ k_explicit_wide(const __grid_constant__ TcDev d, int k, int ja, int jw, int R) {
 // Many cases of one form in one launch: emap[block] = (case, block within the
 // case; -1: the case's mean flow)
 template <int MODE>
-__global__ void __launch_bounds__(32 * EXPLICIT_WARPS, 3)
+__global__ void __launch_bounds__(32 * EXPLICIT_WARPS, MODE == 1 ? 4 : 3)
 k_explicit_b(const TcDev* __restrict__ ds, const int2* __restrict__ emap, int k, int Lc) {
     const int2 m = emap[blockIdx.x];
     const TcDev& d = ds[m.x];

@@ -60,7 +60,7 @@ def parse():
     p.add_argument("--column-groups", type=int, default=0,
                    help="pin the column groups of the step graph (0: chosen by timing)")
     p.add_argument("--line-variant", type=int, default=0,
-                   help="pin the line-kernel variant (0: chosen by timing; the launch shape changes no bits)")
+                   help="pin the line-phase variant (0: chosen by timing; the launch shape changes no bits)")
     p.add_argument("--ztile", type=int, default=0,
                    help="pin the z tile of the z kernels (0: chosen by timing)")
     p.add_argument("--rk-deferral", type=int, default=-1, choices=[-1, 0, 1],
@@ -484,12 +484,13 @@ def torque_summary(series):
             "energy_last": float(series["energy"][-1])}
 
 
-# DRAM bytes per z row of k_rows<double> (Ntheta = 512, Mt = 768): one ncu
-# capture (dram__bytes_read.sum + dram__bytes_write.sum) of the current
-# kernel on the paper workload 129 x 512 x 170, 32895 rows per launch; the
-# per-row traffic does not depend on Nr or Nz.
+# DRAM bytes per z row of the float64 theta rows (Ntheta = 512, Mt = 768): one
+# ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) on the paper
+# workload 129 x 512 x 170, 32895 rows per launch, of the float64 kernel that
+# the fixed-point one replaced (same planes in and out); the per-row traffic
+# does not depend on Nr or Nz.
 ROWS_FP64_BYTES_PER_ROW = {512: (404781824 + 630402816) / 32895}
-ROWS_FP64_CAPTURE_CURRENT = True
+ROWS_FP64_CAPTURE_CURRENT = False
 
 
 def roofline_of(w, prec_name, ph, peaks):
@@ -510,11 +511,13 @@ def roofline_of(w, prec_name, ph, peaks):
                 "peak_source": ("measured FP64 FMA probe (tc_fma_peak) in this run" if prec_name == "fp64"
                                 else "measured FP32 FMA probe (tc_fma_peak) in this run"),
                 "hbm_gbs_of_kernel": a["bytes"] / t / 1e9}
+        if prec_name != "mixed":
+            roof["note"] = "64-bit fixed-point transforms on the integer pipes; the flops are their float64 equivalents"
     else:
         roof = {"bound": "hbm", "achieved": a["bytes"] / t / 1e9, "peak": hbm, "unit": "GB/s",
                 "frac": (a["bytes"] / t / 1e9 / hbm) if hbm else None, "traffic": None,
                 "kernel": dom, "peak_source": "MEASURED_PEAKS.json hbm_gbs (burst)",
-                "note": "the line kernel is float64-issue-bound (ncu); bytes/time is reported against HBM"}
+                "note": "the line phase is float64-issue-bound (ncu); bytes/time is reported against HBM"}
     if dom == "theta_rows_products" and prec_name == "fp64" and w["Ntheta"] in ROWS_FP64_BYTES_PER_ROW:
         rows = w["Nr"] * 3 * w["Nz"] // 2
         scaled = ROWS_FP64_BYTES_PER_ROW[w["Ntheta"]] * rows
@@ -523,8 +526,8 @@ def roofline_of(w, prec_name, ph, peaks):
             roof["traffic"] = scaled
             roof["traffic_source"] = src
         else:
-            roof["traffic_last_capture"] = {"bytes": scaled, "source": src + ", taken before the kernel's "
-                                            "last change (forward plan order, products' scale factor)"}
+            roof["traffic_last_capture"] = {"bytes": scaled, "source": src + ", taken before the transforms "
+                                            "moved to fixed point"}
     roof["phase_ms"] = ph
     return roof
 

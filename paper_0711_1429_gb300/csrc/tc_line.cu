@@ -1287,7 +1287,8 @@ k_solve_shared_b(const TcDev* __restrict__ ds, const int2* __restrict__ bmap, in
 // The explicit rows, four warps a block: warp w of the launch takes chunk w % nch
 // (Lc rows each) of the 32 pairs w / nch, so that the warps of a block mostly share
 // the points at their chunks' ends.  With `mean`, the last block advances the mean
-// flow, which needs the products only.
+// flow, which needs the products only.  Three blocks per SM; the mixed form, with
+// fewer registers, four (five steps of 129x128x128: 7.27 -> 7.01 ms).
 template <int MODE>
 __device__ __forceinline__ void explicit_body(const TcDev& d, int k, int ja, int jw, int Lc, int block) {
     const int nch = (d.Nr - 4 + Lc - 1) / Lc;

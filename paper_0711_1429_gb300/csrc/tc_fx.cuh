@@ -434,7 +434,8 @@ FX_HD int fx_clz(unsigned long long a) {
 #endif
 }
 // fixed point -> bits of the float64 F 2^(eb - 1023), rounded to nearest (values
-// below the normal range become zero)
+// below the normal range become zero, beyond the range infinite: the carry of a
+// rounding at its top ends there by itself)
 FX_HD unsigned long long fx_bits(fx_t F, int eb) {
     const fx_t s = F >> 63;
     const unsigned long long a = (unsigned long long)((F ^ s) - s);
@@ -442,7 +443,8 @@ FX_HD unsigned long long fx_bits(fx_t F, int eb) {
     const int lz = fx_clz(a);
     const unsigned long long m = a << lz;
     const int e = eb + 63 - lz;
-    const unsigned long long b = ((unsigned long long)(unsigned)(e - 1) << 52) + (m >> 11) + ((m >> 10) & 1);
+    const unsigned long long b = e > 2046 ? 0x7ff0000000000000ull
+                                          : ((unsigned long long)(unsigned)(e - 1) << 52) + (m >> 11) + ((m >> 10) & 1);
     return e < 1 ? 0 : b | ((unsigned long long)s & 0x8000000000000000ull);
 }
 // x 2^s, s of either sign

@@ -414,14 +414,13 @@ template <int M, int S> FX_HD int fx_scale(unsigned umax, unsigned usum, int ext
     return fx_headroom<M, S>(emax + 1 + extra, emax + fx_bitlen(usum) - 18);
 }
 #define FX_ZERO 4000   // a scale that makes every value zero
-FX_HD int fx_scale_or_zero(int eb) { return eb < 80 ? FX_ZERO : eb; }
 
 // float64 (as its two words) -> fixed point with scale EB
 FX_HD fx_t fx_from(unsigned hi, unsigned lo, int EB) {
-    const int ex = (int)((hi >> 20) & 0x7ffu);
-    int rs = EB - ex;
+    const int ex = (int)((hi >> 20) & 0x7ffu), normal = ex > 0 ? 1 : 0;     // a subnormal number has exponent 1, no hidden bit
+    int rs = EB - ex - 1 + normal;
     rs = rs > 63 ? 63 : rs;
-    const unsigned mh = (hi & 0xfffffu) | 0x100000u;
+    const unsigned mh = (hi & 0xfffffu) | ((unsigned)normal << 20);
     const unsigned long long m = ((((unsigned long long)mh << 32) | lo) << 10) >> rs;
     const fx_t s = (fx_t)((int)hi >> 31);
     return ((fx_t)m ^ s) - s;
@@ -433,9 +432,9 @@ FX_HD int fx_clz(unsigned long long a) {
     return __builtin_clzll(a);
 #endif
 }
-// fixed point -> bits of the float64 F 2^(eb - 1023), rounded to nearest (values
-// below the normal range become zero, beyond the range infinite: the carry of a
-// rounding at its top ends there by itself)
+// fixed point -> bits of the float64 F 2^(eb - 1023), rounded to nearest over the
+// whole range: subnormal below the normal numbers, infinite beyond the largest (the
+// carry of a rounding at the top of either ends there by itself)
 FX_HD unsigned long long fx_bits(fx_t F, int eb) {
     const fx_t s = F >> 63;
     const unsigned long long a = (unsigned long long)((F ^ s) - s);
@@ -443,9 +442,11 @@ FX_HD unsigned long long fx_bits(fx_t F, int eb) {
     const int lz = fx_clz(a);
     const unsigned long long m = a << lz;
     const int e = eb + 63 - lz;
-    const unsigned long long b = e > 2046 ? 0x7ff0000000000000ull
-                                          : ((unsigned long long)(unsigned)(e - 1) << 52) + (m >> 11) + ((m >> 10) & 1);
-    return e < 1 ? 0 : b | ((unsigned long long)s & 0x8000000000000000ull);
+    unsigned long long b;
+    if ((unsigned)(e - 1) < 2046u) b = ((unsigned long long)(unsigned)(e - 1) << 52) + (m >> 11) + ((m >> 10) & 1);
+    else if (e > 0) b = 0x7ff0000000000000ull;
+    else b = e < -51 ? (unsigned long long)(e == -52) : (m >> (12 - e)) + ((m >> (11 - e)) & 1);
+    return b | ((unsigned long long)s & 0x8000000000000000ull);
 }
 // x 2^s, s of either sign
 FX_HD fx_t fx_shift(fx_t x, int s) { return s >= 0 ? (fx_t)((unsigned long long)x << s) : x >> (s < -63 ? 63 : -s); }

@@ -88,7 +88,7 @@ template <int M, int R> FX_HD constexpr bool fx_dead_leg(int r) {
 }
 
 // Exponents beside the planes: the value of F is F 2^(e - 1023).
-#define FX_NONE (-(1 << 20))    // a column or row of zeros
+#define FX_NONE (-(1 << 20))    // below every exponent: no value at all
 #define FX_BAD (1 << 20)        // one with a NaN or an infinity, or beyond float64
 __device__ __forceinline__ unsigned fx_abs_hi(fx_t F) {      // |F| < (this) 2^32
     const int h = (int)(F >> 32);
@@ -137,7 +137,7 @@ kx_zinv(const __grid_constant__ TcDev d1, const TcDev* __restrict__ ds, const in
         if (!fx_dead_leg<M, R>(r)) sm += fx_mag(fx_hiabs(x[r].x), um >> 20) + fx_mag(fx_hiabs(x[r].y), um >> 20);
     fx_column_reduce<true>(on ? sm : 0u, csm, ct, c);
     __syncthreads();
-    const int EB = fx_scale_or_zero(fx_scale<M, 1>(um, csm[c], 1));
+    const int EB = fx_scale<M, 1>(um, csm[c], 1);
     if (on) {
         fxc v[R];
 #pragma unroll
@@ -175,8 +175,7 @@ kx_zinv(const __grid_constant__ TcDev d1, const TcDev* __restrict__ ds, const in
         out[(size_t)fx_pos<M, NP - 1>(t, r) * Nh] = o;
     }
     if (t == 0)
-        d.zexp[((size_t)f * Nr + rp) * Nh + j] =
-            um >= FX_NONFINITE ? FX_BAD : EB == FX_ZERO ? FX_NONE : EB - 62 + fx_gain<M>() - up;
+        d.zexp[((size_t)f * Nr + rp) * Nh + j] = um >= FX_NONFINITE ? FX_BAD : EB - 62 + fx_gain<M>() - up;
 }
 
 // ---- axial forward: pbuf, pexp -> spectral products, scaled by 1/(Mt Mz) -----------
@@ -467,9 +466,7 @@ kx_rows(const __grid_constant__ TcDev d1, const TcDev* __restrict__ ds, const in
     // exponents of the results: a product of values with exponents a, b (E - 62 +
     // gain each, / 2^64, shifted by hs), the forward gain and the unpacking's 1/2
     const int base = 2 * (fx_gain<M>() - 62) - 1023 + 64 + hs + fx_gain<M>() - 1;
-    auto exponent = [&](int e, bool zero) {
-        return bad || e > 1980 ? FX_BAD : zero || e < -4000 ? FX_NONE : e;
-    };
+    auto exponent = [&](int e) { return bad || e > 1980 ? FX_BAD : e; };
     __syncthreads();
     // ---- forward transforms, two real signals each: role 2 one, the others two ----
     fxc* const pb = reinterpret_cast<fxc*>(d.pbuf) + (size_t)rp * Mz * Nh;
@@ -513,12 +510,11 @@ kx_rows(const __grid_constant__ TcDev d1, const TcDev* __restrict__ ds, const in
         }
         if (t == 0) {
             if (role == 2) {
-                const int e = exponent(base + 2 * Em, em0 == FX_NONE && em1 == FX_NONE);
+                const int e = exponent(base + 2 * Em);
                 if (have0) pe[2 * pes + q0] = e;
                 if (have1) pe[2 * pes + q0 + 1] = e;
             } else if (w1) {
-                pe[k * pes + q0 + role] = k ? exponent(base + Euv + Ew, em0 == FX_NONE || em1 == FX_NONE)
-                                            : exponent(base + 2 * Euv, em0 == FX_NONE);
+                pe[k * pes + q0 + role] = exponent(base + Euv + (k ? Ew : Euv));
             }
         }
     }
@@ -624,7 +620,7 @@ kx_phys(const __grid_constant__ TcDev d, int4 zr) {
     }
     __syncthreads();
     if (!on) return;
-    const int eb = em == FX_NONE ? 0 : EB - 62 + fx_gain<M>();
+    const int eb = EB - 62 + fx_gain<M>();
     const bool bad = em >= FX_BAD;
     auto row = [&](int q) {
         return d.phys + ((size_t)rp * Mz + q / zr.z + zr.x * (q % zr.z / zr.w + zr.y * (q % zr.w))) * M;

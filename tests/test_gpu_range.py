@@ -55,3 +55,23 @@ def test_sums_beyond_the_range_are_infinite(Nt, Nz):
     for got in _both_routes(F, Nt):
         assert np.array_equal(got[over], np.sign(ref[over]) * np.inf)
         assert np.all(np.abs(got[under] * 2.0 ** -8 - ref[under]) <= tol)
+
+
+# Beyond the relative bound: a column of subnormal numbers has the scale of the largest
+# subnormal, so its fixed-point unit is up to 2^-1071 (96 x 48: 2^-1023 2^2 for the
+# value, 2^10 for the sum of up to 72 x 2 of them, 2^-62), and some 2^6 of them round.
+@pytest.mark.parametrize("scale", [2.0 ** -950, 2.0 ** -1000, 2.0 ** -1035, 2.0 ** -1050])
+@pytest.mark.parametrize("Nt,Nz", [(8, 8), (24, 16), (96, 48)])
+def test_tiny_fields_are_not_taken_for_zero(Nt, Nz, scale):
+    Nr, Nh = 9, Nt // 2
+    rng = np.random.default_rng(Nt)
+    F = rng.standard_normal((Nr, Nz, Nh)) + 1j * rng.standard_normal((Nr, Nz, Nh))
+    F[:, Nz // 2], F[:, 0, 0] = 0.0, 0.0
+    F[:, 0, 0] = 0.0
+    for n in range(1, Nz // 2):
+        F[:, Nz - n, 0] = F[:, n, 0].conj()
+    F = (F * scale) / scale * scale                     # rounded to what is stored
+    ref = _phys(F / scale, 3 * Nz // 2, 3 * Nt // 2)
+    tol = 1e-14 * np.abs(ref).max() + 2.0 ** -1065 / scale
+    for got in _both_routes(F, Nt):
+        assert np.abs(got / scale - ref).max() <= tol

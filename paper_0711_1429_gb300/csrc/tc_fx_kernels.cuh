@@ -89,7 +89,7 @@ template <int M, int R> FX_HD constexpr bool fx_dead_leg(int r) {
 
 // Exponents beside the planes: the value of F is F 2^(e - 1023).
 #define FX_NONE (-(1 << 20))    // below every exponent: no value at all
-#define FX_BAD (1 << 20)        // one with a NaN or an infinity, or beyond float64
+#define FX_BAD (1 << 20)        // above every exponent: one with a NaN or an infinity
 __device__ __forceinline__ unsigned fx_abs_hi(fx_t F) {      // |F| < (this) 2^32
     const int h = (int)(F >> 32);
     return (unsigned)(h ^ (h >> 31)) + 1u;
@@ -466,7 +466,7 @@ kx_rows(const __grid_constant__ TcDev d1, const TcDev* __restrict__ ds, const in
     // exponents of the results: a product of values with exponents a, b (E - 62 +
     // gain each, / 2^64, shifted by hs), the forward gain and the unpacking's 1/2
     const int base = 2 * (fx_gain<M>() - 62) - 1023 + 64 + hs + fx_gain<M>() - 1;
-    auto exponent = [&](int e) { return bad || e > 1980 ? FX_BAD : e; };
+    auto exponent = [&](int e) { return bad ? FX_BAD : e; };
     __syncthreads();
     // ---- forward transforms, two real signals each: role 2 one, the others two ----
     fxc* const pb = reinterpret_cast<fxc*>(d.pbuf) + (size_t)rp * Mz * Nh;

@@ -18,7 +18,8 @@ cudaError_t tc_rows_phys_attributes();
     bool tc_fx_rows_##TAG(const TcDev&, const TcDev*, const int2*, int, cudaStream_t);                                  \
     bool tc_fx_phys_##TAG(const TcDev&, int4, cudaStream_t);                                                            \
     bool tc_fx_order_##TAG(int, int4&);                                                                                 \
-    bool tc_fx_attributes_##TAG(int, int, cudaError_t&);
+    bool tc_fx_attributes_##TAG(int, int, cudaError_t&);                                                                \
+    void tc_fx_phys_attributes_##TAG(cudaError_t&);
 FX_GROUP(a) FX_GROUP(b) FX_GROUP(c) FX_GROUP(d)
 #undef FX_GROUP
 
@@ -52,6 +53,15 @@ cudaError_t tc_fx_attributes(int Mtx, int Mzx) {
     tc_fx_attributes_b(Mtx, Mzx, e);
     tc_fx_attributes_c(Mtx, Mzx, e);
     tc_fx_attributes_d(Mtx, Mzx, e);
+    return e;
+}
+
+cudaError_t tc_fx_physical_attributes() {
+    cudaError_t e = cudaSuccess;
+    tc_fx_phys_attributes_a(e);
+    tc_fx_phys_attributes_b(e);
+    tc_fx_phys_attributes_c(e);
+    tc_fx_phys_attributes_d(e);
     return e;
 }
 

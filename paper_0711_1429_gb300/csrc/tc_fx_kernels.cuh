@@ -658,21 +658,24 @@ template <int M> static void fx_launch_phys(const TcDev& d, int4 zr, cudaStream_
 }
 template <int M> static int4 fx_order() { return make_int4(FxPlan<M>::R0, FxPlan<M>::R1, fx_stride<M, 0>(), fx_stride<M, 1>()); }
 // shared-memory opt-in of the kernels of length M that the axial or the theta
-// transforms use
-template <int M> static void fx_attributes(bool rows, bool z, cudaError_t& e) {
+// transforms use, or (phys) those of the physical output in either direction
+template <int M> static void fx_attributes(bool rows, bool z, bool phys, cudaError_t& e) {
     auto set = [&](const void* f, int bytes) {
         const cudaError_t r = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         if (r != cudaSuccess) e = r;
     };
     const int zb = fx_z_columns<M>() * (M + M / 8) * (int)sizeof(fxc);
-    if (z) { set((const void*)kx_zinv<M>, zb); set((const void*)kx_zfwd<M, false>, zb); set((const void*)kx_zfwd<M, true>, zb); }
-    if (rows) { set((const void*)kx_rows<M>, fx_rows_smem<M>()); set((const void*)kx_phys<M>, fx_rows_smem<M>() / 5); }
+    if (z || phys) set((const void*)kx_zinv<M>, zb);
+    if (z) { set((const void*)kx_zfwd<M, false>, zb); set((const void*)kx_zfwd<M, true>, zb); }
+    if (rows) set((const void*)kx_rows<M>, fx_rows_smem<M>());
+    if (rows || phys) set((const void*)kx_phys<M>, fx_rows_smem<M>() / 5);
 }
 #define FX_CASE_Z(M) case M: fx_launch_z<M>(d, ds, ymap, nplanes, which, s, col0, ncols); return true;
 #define FX_CASE_ROWS(M) case M: fx_launch_rows<M>(d, ds, ymap, nplanes, s); return true;
 #define FX_CASE_PHYS(M) case M: fx_launch_phys<M>(d, zr, s); return true;
 #define FX_CASE_ORDER(M) case M: zr = fx_order<M>(); return true;
-#define FX_CASE_ATTR(M) if (Mtx == M || Mzx == M) fx_attributes<M>(Mtx == M, Mzx == M, e);
+#define FX_CASE_ATTR(M) if (Mtx == M || Mzx == M) fx_attributes<M>(Mtx == M, Mzx == M, false, e);
+#define FX_CASE_PHYS_ATTR(M) fx_attributes<M>(false, false, true, e);
 // The launchers of one group of lengths: false for a length of another group.
 #define FX_INSTANTIATE(TAG, LIST)                                                                                        \
     bool tc_fx_z_##TAG(const TcDev& d, const TcDev* ds, const int2* ymap, int nplanes, int which, cudaStream_t s,        \
@@ -684,4 +687,5 @@ template <int M> static void fx_attributes(bool rows, bool z, cudaError_t& e) {
     }                                                                                                                   \
     bool tc_fx_phys_##TAG(const TcDev& d, int4 zr, cudaStream_t s) { switch (d.Mt) { LIST(FX_CASE_PHYS) default: return false; } } \
     bool tc_fx_order_##TAG(int M, int4& zr) { switch (M) { LIST(FX_CASE_ORDER) default: return false; } }                \
-    bool tc_fx_attributes_##TAG(int Mtx, int Mzx, cudaError_t& e) { LIST(FX_CASE_ATTR) return e == cudaSuccess; }
+    bool tc_fx_attributes_##TAG(int Mtx, int Mzx, cudaError_t& e) { LIST(FX_CASE_ATTR) return e == cudaSuccess; }        \
+    void tc_fx_phys_attributes_##TAG(cudaError_t& e) { LIST(FX_CASE_PHYS_ATTR) }

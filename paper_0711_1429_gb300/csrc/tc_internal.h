@@ -171,6 +171,8 @@ void tc_launch_plane_kernel_batch(const TcDev& d0, const TcDev* ds, const int2* 
 void tc_fx_plane_kernel(const TcDev& d, const TcDev* ds, const int2* ymap, int nplanes, int which, cudaStream_t s,
                         int col0, int ncols);
 cudaError_t tc_fx_attributes(int Mtx, int Mzx);
+// that of the physical output's kernels at every planned length
+cudaError_t tc_fx_physical_attributes();
 // physical output of one field through zbuf, zexp and the tables (phx = 1; false, and
 // nothing launched, otherwise)
 bool tc_fx_to_physical(const TcDev& d, const double2* field, cudaStream_t s);

@@ -19,11 +19,9 @@
 // pair of lengths), and as many radial planes as the array holds go through
 // each pair of launches.
 #include <algorithm>
-#include <array>
 #include <cstring>
 #include <map>
 #include <mutex>
-#include <set>
 #include <string>
 #include <utility>
 #include <vector>
@@ -35,6 +33,9 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[TC_NOALLOC_SCRA
 
 bool tc_build_fft_plan(int M, FftPlan& p, std::vector<long double>& re, std::vector<long double>& im, int family);
 void tc_set_error_message(const std::string& s);
+
+__global__ void k_noalloc_twiddles(FftPlan p, double2* tw);
+__global__ void k_noalloc_fx_twiddles(fxw* tw, int M, int st0, int count0, int n1, int st1, int count);
 
 namespace {
 
@@ -89,9 +90,10 @@ bool plans_for(int Mz, int Mt, FftPlan& pz, FftPlan& pt) {
 }
 
 // Device address of the scratch array for the current device (set-up on the
-// first call per device and size: symbol address and the shared-memory opt-in of the
-// transform kernels).
-int scratch_for_current_device(int Mt, int Mz, unsigned char** out) {
+// first call per device: symbol address, and the shared-memory opt-in of the
+// transform kernels of every length, which also loads them, so that a later call
+// of any size can be captured).
+int scratch_for_current_device(unsigned char** out) {
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
@@ -107,21 +109,15 @@ int scratch_for_current_device(int Mt, int Mz, unsigned char** out) {
             return TC_ERR_CUDA;
         }
         e = tc_set_kernel_attributes();
+        if (e == cudaSuccess) e = tc_fx_physical_attributes();
+        cudaFuncAttributes fa;
+        for (const void* f : {(const void*)k_noalloc_twiddles, (const void*)k_noalloc_fx_twiddles})
+            if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, f);
         if (e != cudaSuccess) {
             tc_set_error_message(std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
             return TC_ERR_CUDA;
         }
         g_scratch_dev[dev] = static_cast<unsigned char*>(p);
-    }
-    // the fixed-point kernels' opt-in, once per device and pair of planned lengths
-    static std::set<std::array<int, 3>> ready;
-    if (ready.find({dev, Mt, Mz}) == ready.end()) {
-        e = tc_fx_attributes(Mt, Mz);
-        if (e != cudaSuccess) {
-            tc_set_error_message(std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
-            return TC_ERR_CUDA;
-        }
-        ready.insert({dev, Mt, Mz});
     }
     *out = g_scratch_dev[dev];
     return TC_OK;
@@ -240,7 +236,7 @@ extern "C" int tc_to_physical_noalloc(int Nr, int Ntheta, int Nz, const void* sp
         return TC_ERR_SIZE;
     }
     unsigned char* scratch = nullptr;
-    int rc = scratch_for_current_device(d.Mt, d.Mz, &scratch);
+    int rc = scratch_for_current_device(&scratch);
     if (rc) return rc;
     cudaStream_t s = (cudaStream_t)cuda_stream;
     // Every call rewrites the twiddles, and the z transform fully writes each

@@ -410,12 +410,8 @@ __device__ __forceinline__ void rk_memory_row(const TcDev& d, const double* __re
     H[2 * (size_t)jr * d.npairs] = fma(hdt, acc, H[2 * (size_t)jr * d.npairs]);
 }
 // The rows centred on i0 <= i < i1 (v: 2 .. Nr - 3; the one-sided eta rows 1 and
-// Nr - 2 with their neighbours).  BAND: the eta band is formed here instead of read,
-// with the table's own operations, where the float64 pipe has time to spare but not
-// the memory: beside the mixed form's theta rows.
-template <bool BAND = false>
-__device__ __forceinline__ void rk_memory_rows(const TcDev& d, int k, int pair, int comp, int i0, int i1, double m = 0.0,
-                                               double al = 0.0) {
+// Nr - 2 with their neighbours).
+__device__ __forceinline__ void rk_memory_rows(const TcDev& d, int k, int pair, int comp, int i0, int i1) {
     const int N = d.Nr, kn = (k + 1) % 3;
     const size_t P2 = 2 * (size_t)d.npairs;
     const double hdt = (d.rk_beta[k] + d.rk_alpha[kn]) * d.dt, hdtnu = hdt * d.nu;
@@ -427,30 +423,14 @@ __device__ __forceinline__ void rk_memory_rows(const TcDev& d, int k, int pair, 
     if (i0 >= i1) return;
     double xv[5], xe[5];
     for (int s = 0; s < 4; ++s) { xv[s + 1] = v[(i0 - 2 + s) * P2]; xe[s + 1] = e[(i0 - 2 + s) * P2]; }
-    double k2[5];
-    if constexpr (BAND)
-        for (int s = 0; s < 4; ++s) k2[s + 1] = k2_at(m, al, d.rinv[i0 - 2 + s]);
-    auto eta_row = [&](int j) {
-        if constexpr (BAND) {
-            double acc = 0.0;
-            for (int s = 0; s < 5; ++s) acc = fma(fma(-d.d0[j * 5 + s], k2[s], d.l2[j * 5 + s]), xe[s], acc);
-            He[(size_t)j * P2] = fma(hdtnu, acc, He[(size_t)j * P2]);
-        } else {
-            rk_memory_row(d, d.tab_le, He, pair, j, xe, hdtnu);
-        }
-    };
     for (int i = i0; i < i1; ++i) {
         for (int s = 0; s < 4; ++s) { xv[s] = xv[s + 1]; xe[s] = xe[s + 1]; }
-        if constexpr (BAND) {
-            for (int s = 0; s < 4; ++s) k2[s] = k2[s + 1];
-            k2[4] = k2_at(m, al, d.rinv[i + 2]);
-        }
         xv[4] = v[(i + 2) * P2];
         xe[4] = e[(i + 2) * P2];
         rk_memory_row(d, d.tab_lv, Hv, pair, i, xv, hdt);
-        eta_row(i);
-        if (i == 2) eta_row(1);
-        if (i == N - 3) eta_row(N - 2);
+        rk_memory_row(d, d.tab_le, He, pair, i, xe, hdtnu);
+        if (i == 2) rk_memory_row(d, d.tab_le, He, pair, 1, xe, hdtnu);
+        if (i == N - 3) rk_memory_row(d, d.tab_le, He, pair, N - 2, xe, hdtnu);
     }
 }
 
@@ -1061,18 +1041,49 @@ constexpr long long WIDE_GROUPS = 8 * 152;
 static bool solve_wide(long long groups, int Nr) { return groups < WIDE_GROUPS && solve_smem(Nr) <= 200 * 1024; }
 
 // The implicit part of the next RK memory (rk_memory_row) for the pairs of
-// the columns ja .. ja + jw - 1, after a k_solve of substep k launched with NOH:
-// one thread per pair and component walks its radial line.  It needs only the
-// results of that kernel, so it can run beside the next substep's plane phase.
+// the columns ja .. ja + jw - 1, after a k_solve of substep k launched with NOH.  It
+// needs only the results of that kernel, so it can run beside the next substep's
+// plane phase.
 // Grid-stride over the pairs: launched beside the theta rows it runs in few
 // blocks (four per SM), so that it takes mostly what the rows leave free.
-__global__ void __launch_bounds__(128) k_rk_memory(TcDev d, int k, int ja, int jw) {
-    const int n = 2 * d.Nz * jw;
+// What bounds it there is the float64 pipe, so a thread walks a pair's whole line with
+// both components, and the eta band, formed with the table's own operations (where the
+// pipe has more time to spare than the memory), serves both: 32 operations a point
+// against 40 with a lane per component, 2.31 -> 2.06 ms alone at 257x512x512.  Step of
+// the mixed form there: 38.9 -> 37.25 ms (solves with the RK memory in them: 39.0; with
+// the band read here: 38.8); of 129x512x170: 7.66 -> 7.45 (7.73).
+__global__ void __launch_bounds__(128) k_rk_memory(const __grid_constant__ TcDev d, int k, int ja, int jw) {
+    const int N = d.Nr, kn = (k + 1) % 3, n = d.Nz * jw;
+    const size_t P = d.npairs;
+    const double hdt = (d.rk_beta[k] + d.rk_alpha[kn]) * d.dt, hdtnu = hdt * d.nu;
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += gridDim.x * blockDim.x) {
         int pair;
         double m, al;
         long long partner;
-        if (line_pair(d, ja, jw, idx >> 1, pair, m, al, partner)) rk_memory_rows<true>(d, k, pair, idx & 1, 0, d.Nr, m, al);
+        if (!line_pair(d, ja, jw, idx, pair, m, al, partner)) continue;
+        const double2 *v = d.v + pair, *e = d.eta + pair;
+        double2 xv[5], xe[5];
+        double k2[5];
+        for (int s = 0; s < 4; ++s) { xv[s + 1] = v[s * P]; xe[s + 1] = e[s * P]; k2[s + 1] = k2_at(m, al, d.rinv[s]); }
+        auto eta_row = [&](int j) {
+            double2 acc = cz();
+            for (int s = 0; s < 5; ++s) acc = caxpy(acc, fma(-d.d0[j * 5 + s], k2[s], d.l2[j * 5 + s]), xe[s]);
+            double2* H = d.He + (size_t)j * P + pair;
+            *H = caxpy(*H, hdtnu, acc);
+        };
+        for (int i = 2; i < N - 2; ++i) {
+            for (int s = 0; s < 4; ++s) { xv[s] = xv[s + 1]; xe[s] = xe[s + 1]; k2[s] = k2[s + 1]; }
+            xv[4] = v[(i + 2) * P];
+            xe[4] = e[(i + 2) * P];
+            k2[4] = k2_at(m, al, d.rinv[i + 2]);
+            double2 acc = cz();
+            for (int s = 0; s < 5; ++s) acc = caxpy(acc, TAB(d.tab_lv, 0, i, s), xv[s]);
+            double2* H = d.Hv + (size_t)i * P + pair;
+            *H = caxpy(*H, hdt, acc);
+            eta_row(i);
+            if (i == 2) eta_row(1);
+            if (i == N - 3) eta_row(N - 2);
+        }
     }
 }
 
@@ -1646,7 +1657,7 @@ void tc_launch_line_chunk(const TcDev& d, int k, cudaStream_t s, int ja, int jw,
 void tc_launch_line_phase(const TcDev& d, int k, cudaStream_t s, bool mean) { tc_launch_line_chunk(d, k, s, 0, d.Nh, mean, false); }
 
 void tc_launch_rk_memory(const TcDev& d, int k, cudaStream_t s, int ja, int jw, bool background) {
-    int blocks = (2 * d.Nz * jw + 127) / 128;
+    int blocks = (d.Nz * jw + 127) / 128;
     if (background) {
         static int sms = 0;
         if (!sms) {

@@ -130,3 +130,32 @@ def test_products_at_the_ends_of_the_range(Nt, Nz, peak):
             norm = max(np.sqrt(np.sum(p[r] ** 2) / (Mz * Mt)), np.linalg.norm(want[r]))
             tol = 2e-15 * norm + 2.0 ** (-1073 - 2 * peak) * np.sqrt(Nz * Nh)
             assert np.linalg.norm(_times(got[k, r], -2 * peak) - want[r]) <= tol, (k, r)
+
+
+def test_products_of_a_spot():
+    """Velocities that fall off in z by many orders from a spot: the theta rows of a plane
+    share one scale, so the quiet rows keep fewer bits than the spot's, and the
+    products, sums over all rows, must not show it (bound as in the tests of fields
+    that fill the box)."""
+    Nr, Nt, Nz = 9, 48, 96
+    Nh, Mz, Mt = Nt // 2, 3 * Nz // 2, 3 * Nt // 2
+    rng = np.random.default_rng(3)
+    n = np.minimum(np.arange(Nz), Nz - np.arange(Nz))
+    spot = np.exp(-(n / 8.0) ** 2)[:, None] * np.exp(-np.arange(Nh) / 6.0)         # all modes in phase at z = 0
+    s = np.linspace(-1, 1, Nr)[:, None, None]
+    a = 1 + 0.1 * rng.standard_normal((Nr, 1, Nh)) + 0.1j * rng.standard_normal((Nr, 1, Nh))
+    a[:, :, 0] = 0.0                                    # (the slot (0, 0) is not a field's, and its lack is not local)
+    v, e = 1e-2 * (1 - s * s) ** 2 * spot * a, 3e-2 * (1 - s * s) * spot * a.imag
+    for F in (v, e):
+        F[:, Nz // 2] = 0.0
+    f, got = _products(v.astype(complex), e.astype(complex), Nt, tc.TC_PREC_FP64)
+    u, v_, w = (_phys(F, Mz, Mt) for F in f)
+    rows = np.abs(v_[Nr // 2]).max(axis=1)
+    assert rows.min() < 1e-6 * rows.max()
+    for k, p in enumerate((u * u - v_ * v_, u * v_, u * w, v_ * w, w * w - v_ * v_)):
+        S = np.fft.rfft2(p, axes=(1, 2))[:, :, :Nh] / (Mz * Mt)
+        want = np.zeros((Nr, Nz, Nh), dtype=complex)
+        want[:, :Nz // 2], want[:, Nz // 2 + 1:] = S[:, :Nz // 2], S[:, Mz - Nz // 2 + 1:]
+        for r in range(Nr):
+            norm = max(np.sqrt(np.sum(p[r] ** 2) / (Mz * Mt)), np.linalg.norm(want[r]))
+            assert np.linalg.norm(got[k, r] - want[r]) <= 2e-15 * norm, (k, r)

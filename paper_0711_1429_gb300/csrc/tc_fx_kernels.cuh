@@ -27,10 +27,10 @@
 #include <type_traits>
 
 __device__ __forceinline__ unsigned fx_hiabs(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
-__device__ __forceinline__ fx_t fx_of(double x, int EB) {
-    return fx_from((unsigned)__double2hiint(x), (unsigned)__double2loint(x), EB);
+template <bool SUB> __device__ __forceinline__ fx_t fx_of(double x, int EB) {
+    return fx_from<SUB>((unsigned)__double2hiint(x), (unsigned)__double2loint(x), EB);
 }
-__device__ __forceinline__ double fx_to(fx_t F, int eb) { return __longlong_as_double((long long)fx_bits(F, eb)); }
+template <bool RANGE> __device__ __forceinline__ double fx_to(fx_t F, int eb) { return __longlong_as_double((long long)fx_bits<RANGE>(F, eb)); }
 __device__ __forceinline__ double fx_nan() { return __longlong_as_double(0x7ff8000000000000ll); }
 __device__ __forceinline__ unsigned umax2(unsigned a, unsigned b) { return a > b ? a : b; }
 // barrier of one role's threads (barriers 1 .. 3; 0 is the block's)
@@ -140,11 +140,15 @@ kx_zinv(const __grid_constant__ TcDev d1, const TcDev* __restrict__ ds, const in
     const int EB = fx_scale<M, 1>(um, csm[c], 1);
     if (on) {
         fxc v[R];
+        auto convert = [&](auto sub) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            v[r].x = v[r].y = 0;
-            if (!fx_dead_leg<M, R>(r)) { v[r].x = fx_of(x[r].x, EB); v[r].y = fx_of(x[r].y, EB); }
-        }
+            for (int r = 0; r < R; ++r) {
+                v[r].x = v[r].y = 0;
+                if (!fx_dead_leg<M, R>(r)) { v[r].x = fx_of<sub.value>(x[r].x, EB); v[r].y = fx_of<sub.value>(x[r].y, EB); }
+            }
+        };
+        if (EB >= FX_SCALE_NORMAL) convert(std::false_type());
+        else convert(std::true_type());
         fx_butterfly<M, 1, 0>(v, t, d.twx_z);
         fx_put<M, 0>(v, col, t, lct);
     }
@@ -261,16 +265,20 @@ kx_zfwd(const __grid_constant__ TcDev d1, const TcDev* __restrict__ ds, const in
             out[(size_t)s * Nh] = e;
         } else out[(size_t)s * Nh] = o;
     };
+    auto store = [&](auto range) {          // with the ends of the float64 range and the mark, or without
 #pragma unroll
-    for (int r = 0; r < RL; ++r) {
-        if (fx_dead_leg<M, RL>(r)) continue;
-        const int q = fx_pos<M, 0>(t, r);
-        const int s = q < Nz / 2 ? q : (q > M - Nz / 2 ? Nz - (M - q) : -1);
-        if (s < 0) continue;
-        double2 o = make_double2(fx_to(z[r].x, eb), fx_to(z[r].y, eb));
-        if (bad) o.x = o.y = fx_nan();
-        put(s, o);
-    }
+        for (int r = 0; r < RL; ++r) {
+            if (fx_dead_leg<M, RL>(r)) continue;
+            const int q = fx_pos<M, 0>(t, r);
+            const int s = q < Nz / 2 ? q : (q > M - Nz / 2 ? Nz - (M - q) : -1);
+            if (s < 0) continue;
+            double2 o = make_double2(fx_to<range.value>(z[r].x, eb), fx_to<range.value>(z[r].y, eb));
+            if (range.value && bad) o.x = o.y = fx_nan();
+            put(s, o);
+        }
+    };
+    if (fx_normal(eb) && !bad) store(std::false_type());
+    else store(std::true_type());
     if (t == 0) put(Nz / 2, make_double2(0.0, 0.0));       // axial Nyquist slot
 }
 
@@ -627,11 +635,15 @@ kx_phys(const __grid_constant__ TcDev d, int4 zr) {
     };
     double* o0 = row(have0 ? q0 : 0);
     double* o1 = row(have1 ? q0 + 1 : 0);
-    for (int p = t; p < M; p += T) {
-        const fxc a = col[fx_pad(p)];
-        if (have0) o0[p] = bad ? fx_nan() : fx_to(a.x, eb);
-        if (have1) o1[p] = bad ? fx_nan() : fx_to(a.y, eb);
-    }
+    auto store = [&](auto range) {          // as in kx_zfwd
+        for (int p = t; p < M; p += T) {
+            const fxc a = col[fx_pad(p)];
+            if (have0) o0[p] = range.value && bad ? fx_nan() : fx_to<range.value>(a.x, eb);
+            if (have1) o1[p] = range.value && bad ? fx_nan() : fx_to<range.value>(a.y, eb);
+        }
+    };
+    if (fx_normal(eb) && !bad) store(std::false_type());
+    else store(std::true_type());
 }
 
 // ---- host launchers ----------------------------------------------------------

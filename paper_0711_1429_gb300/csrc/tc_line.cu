@@ -1089,37 +1089,61 @@ __global__ void __launch_bounds__(128) k_rk_memory(const __grid_constant__ TcDev
 
 // ---------------------------------------------------------------------------
 // Initial RK memory H_1 = (M + alpha_1 dt L) x for v and eta, and u, w, as k_solve
-// after its solves: the rows i0 <= i < i1 of H_1.
-__device__ __forceinline__ void init_rows(const TcDev& d, int pair, int comp, double m, double al, int i0, int i1) {
+// after its solves: the rows i0 <= i < i1 of H_1, both components by one thread, since
+// the bands cost more than the sums with them.  The one-sided eta rows 1 and Nr - 2 go
+// with their neighbours.
+__device__ __forceinline__ void init_rows(const TcDev& d, int pair, double m, double al, int i0, int i1) {
     const int N = d.Nr;
-    const size_t P = d.npairs, P2 = 2 * P, o = 2 * (size_t)pair + comp;
+    const size_t P = d.npairs;
     const double adt = d.rk_alpha[0] * d.dt;
-    const double *v = reinterpret_cast<const double*>(d.v) + o, *e = reinterpret_cast<const double*>(d.eta) + o;
-    double *Hv = reinterpret_cast<double*>(d.Hv) + o, *He = reinterpret_cast<double*>(d.He) + o;
+    const double2 *v = d.v + pair, *e = d.eta + pair;
+    double2 *Hv = d.Hv + pair, *He = d.He + pair;
+    if (i0 == 0) Hv[0] = Hv[P] = He[0] = cz();
+    if (i1 == N) Hv[(size_t)(N - 2) * P] = Hv[(size_t)(N - 1) * P] = He[(size_t)(N - 1) * P] = cz();
+    i0 = i0 < 2 ? 2 : i0;
+    i1 = i1 > N - 2 ? N - 2 : i1;
+    if (i0 >= i1) return;
+    double c[5], c1[5], k2[5];                  // 1/k^2, its derivative and k^2 at the row's points
+    double2 xv[5], xe[5];
+    auto point = [&](int i) {
+        for (int s = 0; s < 4; ++s) { c[s] = c[s + 1]; c1[s] = c1[s + 1]; k2[s] = k2[s + 1]; xv[s] = xv[s + 1]; xe[s] = xe[s + 1]; }
+        const size_t o = (size_t)i * P;
+        const double ri = d.rinv[i];
+        c[4] = d.tab_c[o + pair];
+        c1[4] = d.tab_c1 ? d.tab_c1[o + pair] : coef_at(d.r[i], ri, m, al).c1;
+        k2[4] = al * al + m * m * ri * ri;
+        xv[4] = v[o];
+        xe[4] = e[o];
+    };
+    auto eta_row = [&](int j) {
+        double2 h = cz();
+        for (int s = 0; s < 5; ++s) {
+            const double L5 = d.nu * (d.l2[j * 5 + s] - d.d0[j * 5 + s] * k2[s]);
+            h = caxpy(h, d.d0[j * 5 + s] + adt * L5, xe[s]);
+        }
+        He[(size_t)j * P] = h;
+    };
+    for (int i = i0 - 2; i < i0 + 2; ++i) point(i);
     for (int j = i0; j < i1; ++j) {
-        double hv = 0.0, he = 0.0;
-        if (j >= 2 && j <= N - 3) {
-            // mass band M = d0 - l2 c + l1 c' from the c, c' tables
-            for (int s = 0; s < 5; ++s) {
-                const size_t i = j - 2 + s;
-                const double M5 = d.d0[j * 5 + s] - d.l2[j * 5 + s] * d.tab_c[i * P + pair] + d.l1[j * 5 + s] * (d.tab_c1 ? d.tab_c1[i * P + pair] : coef_at(d.r[i], d.rinv[i], m, al).c1);
-                hv = fma(M5 + adt * TAB(d.tab_lv, 0, j, s), v[i * P2], hv);
-            }
+        point(j + 2);
+        double2 h = cz();
+        for (int s = 0; s < 5; ++s) {           // mass band M = d0 - l2 c + l1 c'
+            const double M5 = d.d0[j * 5 + s] - d.l2[j * 5 + s] * c[s] + d.l1[j * 5 + s] * c1[s];
+            h = caxpy(h, M5 + adt * TAB(d.tab_lv, 0, j, s), xv[s]);
         }
-        if (j >= 1 && j <= N - 2) {
-            const size_t st = d.start[j];
-            for (int s = 0; s < 5; ++s) {
-                const double ri = d.rinv[st + s];
-                const double L5 = d.nu * (d.l2[j * 5 + s] - d.d0[j * 5 + s] * (al * al + m * m * ri * ri));
-                he = fma(d.d0[j * 5 + s] + adt * L5, e[(st + s) * P2], he);
-            }
-        }
-        Hv[(size_t)j * P2] = hv;
-        He[(size_t)j * P2] = he;
+        Hv[(size_t)j * P] = h;
+        eta_row(j);
+        if (j == 2) eta_row(1);
+        if (j == N - 3) eta_row(N - 2);
     }
 }
+// One warp solves for Dv, the others take the rows of H_1.  Bound by the float64 pipe
+// (94 operations a pair and row).  257x512x512: 6.16 ms with four warps (two: 6.37; a
+// lane per component of a row, which formed the bands twice and, in the double-float
+// form, c' five times a row: 9.1 and in that form 15.4, now 6.94); 129x512x170: 1.63 ->
+// 1.06 and 2.62 -> 1.20; 129x128x128, eight warps: 0.36 -> 0.27 and 0.59 -> 0.31.
 template <int WARPS>
-__global__ void __launch_bounds__(32 * WARPS, WARPS > 2 ? 2 : 12) k_init(const __grid_constant__ TcDev d) {
+__global__ void __launch_bounds__(32 * WARPS, WARPS > 4 ? 2 : 4) k_init(const __grid_constant__ TcDev d) {
     const int warp = threadIdx.x >> 5, comp = threadIdx.x & 1;
     int pair = 0;
     double m = 0.0, al = 0.0;
@@ -1132,7 +1156,10 @@ __global__ void __launch_bounds__(32 * WARPS, WARPS > 2 ? 2 : 12) k_init(const _
     __syncthreads();
     if (act) {
         if (warp == 0) derivative_solve(d, t, S);
-        else init_rows(d, pair, comp, m, al, (warp - 1) * N / (WARPS - 1), warp * N / (WARPS - 1));
+        else {                              // the pair's two lanes take half of the rows each
+            const int w = 2 * (warp - 1) + comp;
+            init_rows(d, pair, m, al, w * N / (2 * WARPS - 2), (w + 1) * N / (2 * WARPS - 2));
+        }
     }
     __syncthreads();
     if (act) velocity_rows(d, t, pair, comp, m, al, partner, S, warp * N / WARPS, (warp + 1) * N / WARPS);
@@ -1725,6 +1752,6 @@ cudaError_t tc_set_line_kernel_attributes() {
 void tc_launch_init_state(const TcDev& d, cudaStream_t s) {
     const int half = (d.npairs + 15) / 16;
     if (half < WIDE_GROUPS) k_init<8><<<half, 256, 0, s>>>(d);
-    else k_init<2><<<half, 64, 0, s>>>(d);
+    else k_init<4><<<half, 32 * 4, 0, s>>>(d);
     k_mean_init<<<1, 256, 0, s>>>(d);
 }

@@ -41,3 +41,18 @@ def test_launch_plans_change_no_bits_at_many_pairs(Nr, prec):
             g = run(planned(groups, deferral))
             for k in ref:
                 assert np.array_equal(g[k], ref[k]), (groups, deferral, k)
+
+
+@pytest.mark.parametrize("Nr", [9, 37, 282])
+@pytest.mark.parametrize("prec", [tc.TC_PREC_FP64, tc.TC_PREC_MIXED, tc.TC_PREC_DF64])
+def test_few_pairs_give_finite_fields_that_are_not_zero(Nr, prec):
+    """(The comparison of few and many pairs elsewhere would hold for zeros too.)"""
+    Nt, Nz = 12, 14
+    v, e = inputs(Nr, Nt, Nz, 0.8, 3 + Nr, "box", 1e-2, jmax=Nt // 4, nmax=Nz // 4)
+    h = gpu_case(Nr, Nt, Nz, 0.8, 300.0, -20.0, 2e-3, v=v, eta=e, precision=prec)
+    try:
+        tc.tc_step(h, 2)
+        for k, x in gpu_state(h, Nr, Nz, Nt // 2).items():
+            assert np.all(np.isfinite(x)) and np.any(x != 0.0), k
+    finally:
+        tc.tc_destroy(h)

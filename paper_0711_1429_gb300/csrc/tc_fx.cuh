@@ -415,15 +415,15 @@ template <int M, int S> FX_HD int fx_scale(unsigned umax, unsigned usum, int ext
 }
 #define FX_ZERO 4000   // a scale that makes every value zero
 
-// float64 (as its two words) -> fixed point with scale EB.  Subnormal numbers have
-// exponent 1 and no hidden bit; with a scale of at least FX_SCALE_NORMAL they and zero
-// lie below the last bit anyway, and SUB = false leaves the distinction out (same bits).
-constexpr int FX_SCALE_NORMAL = 80;
-template <bool SUB = true> FX_HD fx_t fx_from(unsigned hi, unsigned lo, int EB) {
-    const int ex = (int)((hi >> 20) & 0x7ffu), normal = !SUB || ex > 0 ? 1 : 0;
-    int rs = EB - ex - 1 + normal;
+// float64 (as its two words) -> fixed point with scale EB; subnormal numbers have exponent
+// 1 and no hidden bit: the upper word less e - 1 in the exponent field has the hidden bit
+// where there is one.  (Two instructions a value; a branch to another conversion for the
+// columns that need it cost the axial inverse 16 registers.)
+FX_HD fx_t fx_from(unsigned hi, unsigned lo, int EB) {
+    const int ex = (int)((hi >> 20) & 0x7ffu), e = ex < 1 ? 1 : ex;
+    int rs = EB - e;
     rs = rs > 63 ? 63 : rs;
-    const unsigned mh = (hi & 0xfffffu) | ((unsigned)normal << 20);
+    const unsigned mh = (hi & 0x7fffffffu) - ((unsigned)(e - 1) << 20);
     const unsigned long long m = ((((unsigned long long)mh << 32) | lo) << 10) >> rs;
     const fx_t s = (fx_t)((int)hi >> 31);
     return ((fx_t)m ^ s) - s;

@@ -27,8 +27,8 @@
 #include <type_traits>
 
 __device__ __forceinline__ unsigned fx_hiabs(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
-template <bool SUB> __device__ __forceinline__ fx_t fx_of(double x, int EB) {
-    return fx_from<SUB>((unsigned)__double2hiint(x), (unsigned)__double2loint(x), EB);
+__device__ __forceinline__ fx_t fx_of(double x, int EB) {
+    return fx_from((unsigned)__double2hiint(x), (unsigned)__double2loint(x), EB);
 }
 template <bool RANGE> __device__ __forceinline__ double fx_to(fx_t F, int eb) { return __longlong_as_double((long long)fx_bits<RANGE>(F, eb)); }
 __device__ __forceinline__ double fx_nan() { return __longlong_as_double(0x7ff8000000000000ll); }
@@ -140,15 +140,11 @@ kx_zinv(const __grid_constant__ TcDev d1, const TcDev* __restrict__ ds, const in
     const int EB = fx_scale<M, 1>(um, csm[c], 1);
     if (on) {
         fxc v[R];
-        auto convert = [&](auto sub) {
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                v[r].x = v[r].y = 0;
-                if (!fx_dead_leg<M, R>(r)) { v[r].x = fx_of<sub.value>(x[r].x, EB); v[r].y = fx_of<sub.value>(x[r].y, EB); }
-            }
-        };
-        if (EB >= FX_SCALE_NORMAL) convert(std::false_type());
-        else convert(std::true_type());
+        for (int r = 0; r < R; ++r) {
+            v[r].x = v[r].y = 0;
+            if (!fx_dead_leg<M, R>(r)) { v[r].x = fx_of(x[r].x, EB); v[r].y = fx_of(x[r].y, EB); }
+        }
         fx_butterfly<M, 1, 0>(v, t, d.twx_z);
         fx_put<M, 0>(v, col, t, lct);
     }

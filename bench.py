@@ -484,15 +484,6 @@ def torque_summary(series):
             "energy_last": float(series["energy"][-1])}
 
 
-# DRAM bytes per z row of the float64 theta rows (Ntheta = 512, Mt = 768): one
-# ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) on the paper
-# workload 129 x 512 x 170, 32895 rows per launch, of the float64 kernel that
-# the fixed-point one replaced (same planes in and out); the per-row traffic
-# does not depend on Nr or Nz.
-ROWS_FP64_BYTES_PER_ROW = {512: (404781824 + 630402816) / 32895}
-ROWS_FP64_CAPTURE_CURRENT = False
-
-
 def roofline_of(w, prec_name, ph, peaks):
     alg = algorithmic(w, prec_name)
     dom = max(ph, key=ph.get)
@@ -504,30 +495,19 @@ def roofline_of(w, prec_name, ph, peaks):
     hbm = meas_peaks.get("hbm_gbs")
     a = alg[dom]
     t = ph[dom] * 1e-3
-    if a["flops"] is not None:
-        pk = peaks["fp64_tflops"] if prec_name == "fp64" else peaks["fp32_tflops"]
+    if a["flops"] is not None and prec_name == "mixed":
+        pk = peaks["fp32_tflops"]
         roof = {"bound": "alu", "achieved": a["flops"] / t / 1e12, "peak": pk, "unit": "TFLOP/s",
                 "frac": a["flops"] / t / 1e12 / pk, "traffic": None, "kernel": dom,
-                "peak_source": ("measured FP64 FMA probe (tc_fma_peak) in this run" if prec_name == "fp64"
-                                else "measured FP32 FMA probe (tc_fma_peak) in this run"),
+                "peak_source": "measured FP32 FMA probe (tc_fma_peak) in this run",
                 "hbm_gbs_of_kernel": a["bytes"] / t / 1e9}
-        if prec_name != "mixed":
-            roof["note"] = "64-bit fixed-point transforms on the integer pipes; the flops are their float64 equivalents"
     else:
+        note = ("the line phase is float64-issue-bound (ncu)" if a["flops"] is None else
+                "64-bit fixed-point transforms, bound by integer issue (ncu), for which no flop rate is a roofline")
         roof = {"bound": "hbm", "achieved": a["bytes"] / t / 1e9, "peak": hbm, "unit": "GB/s",
                 "frac": (a["bytes"] / t / 1e9 / hbm) if hbm else None, "traffic": None,
                 "kernel": dom, "peak_source": "MEASURED_PEAKS.json hbm_gbs (burst)",
-                "note": "the line phase is float64-issue-bound (ncu); bytes/time is reported against HBM"}
-    if dom == "theta_rows_products" and prec_name == "fp64" and w["Ntheta"] in ROWS_FP64_BYTES_PER_ROW:
-        rows = w["Nr"] * 3 * w["Nz"] // 2
-        scaled = ROWS_FP64_BYTES_PER_ROW[w["Ntheta"]] * rows
-        src = "ncu dram bytes per row of k_rows<double> on paper-129x512x170, scaled by rows"
-        if ROWS_FP64_CAPTURE_CURRENT:
-            roof["traffic"] = scaled
-            roof["traffic_source"] = src
-        else:
-            roof["traffic_last_capture"] = {"bytes": scaled, "source": src + ", taken before the transforms "
-                                            "moved to fixed point"}
+                "note": note + "; bytes/time is reported against HBM"}
     roof["phase_ms"] = ph
     return roof
 

@@ -67,8 +67,9 @@ enum { TC_SPECTRAL = 0, TC_PHYSICAL = 1 };
 enum {
     TC_PREC_FP64 = 0,       /* every step in float64, the transforms and products
                                in 64-bit fixed point with one scale per
-                               transform (error below float64's) where the
-                               padded lengths are at most 1536 */
+                               transform (error below float64's, range that of
+                               float64) where the padded lengths are at most
+                               1536 */
     TC_PREC_MIXED = 1,      /* FFTs, products and explicit radial rows in
                                float32, their continuity term in double-float;
                                banded solves, RK memory, reconstruction and

@@ -368,9 +368,9 @@ void free_all(tc_handle* h) {
     h->allocs.clear();
 }
 
-// Tile autotuner: candidate azimuthal tiles of the z kernels and block sizes
-// of the line phase are timed on the (zero) initial state, which they leave
-// unchanged, and the fastest pair is kept for the shape class (Nr, Ntheta,
+// Tile autotuner: candidate azimuthal tiles of the z kernels and rows per warp
+// of the explicit rows are timed on the (zero) initial state, whose fields are zeroed
+// again afterwards, and the fastest pair is kept for the shape class (Nr, Ntheta,
 // Nz, precision).  The choice changes no arithmetic.
 std::mutex g_tune_mu;
 std::map<std::array<int, 4>, std::pair<int, int>> g_tune;

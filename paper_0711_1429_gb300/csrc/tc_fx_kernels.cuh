@@ -17,9 +17,9 @@
 // 768-point transform, half of them in the twiddles), at 40 to 60% of the issue
 // rate between barriers and loads, where the float64 transforms they replace kept
 // the float64 pipe 92% busy.  Per substep of 257x512x512 in the float64 form: axial
-// inverse 6.25 -> 1.61 ms, theta rows 30.96 -> 7.91, axial forward 10.60 -> 2.99; of
-// 129x512x170 (axial length 255, now 256): 1.99 -> 0.27, 5.18 -> 1.33, 4.29 -> 0.58;
-// in the double-float form there 1.04 -> 0.27, 2.15 -> 1.34, 1.63 -> 0.66.
+// inverse 6.25 -> 1.61 ms, theta rows 30.96 -> 7.83, axial forward 10.60 -> 2.93; of
+// 129x512x170 (axial length 255, now 256): 1.99 -> 0.27, 5.18 -> 1.32, 4.29 -> 0.57;
+// in the double-float form there 1.04 -> 0.27, 2.15 -> 1.32, 1.63 -> 0.65.
 #pragma once
 #include "tc_fx.cuh"
 #include "tc_internal.h"

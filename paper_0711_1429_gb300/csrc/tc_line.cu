@@ -299,7 +299,8 @@ __global__ void __launch_bounds__(128) k_setup(TcDev d) {
 // eighth of the operations, are serial in r.  Per substep, line phase of the
 // float64 form before and now: 33x16x16 333 -> 45 us, 64x32x64 684 -> 82,
 // 129x128x128 1118 -> 536, 129x512x170 2897 -> 2400, 257x512x512 15.5 -> 13.5 ms; of
-// the mixed form: 129x128x128 923 -> 350 us, 257x512x512 8.7 -> 8.1 ms.
+// the mixed form: 129x128x128 923 -> 350 us, 257x512x512 7.9 (the best of that kernel's
+// launch shapes) -> 8.0 ms.
 //
 // Explicit rows: sums over the 5 stencil points of d0 . A + l1 . B (+ l2 . C for
 // v), where A, B, C are pointwise "inner" functions of the products and of u, v, w
@@ -400,9 +401,9 @@ struct RowTables { const double *d0, *l1, *dsol, *rinv; };   // the case's own, 
 // Implicit part of the next RK memory on row jr (SMR91 low storage):
 // H_(k+1) += (beta_k + alpha_(k+1)) dt L x^(k+1), with L the band of row jr from the
 // per-pair table, applied to the window x of x^(k+1) on the row's five stencil
-// points.  k_solve calls it after its solves; the deferred form (k_rk_memory)
-// calls it after a k_solve that left it out, with the same operands, so both give
-// the same bits.
+// points.  k_solve calls it after its solves; the deferred form (k_rk_memory), after
+// a k_solve that left it out, has the same operations on the same operands, so both
+// give the same bits.
 __device__ __forceinline__ void rk_memory_row(const TcDev& d, const double* __restrict__ tab, double* H, int pair, int jr,
                                               const double* x, double hdt) {
     double acc = 0.0;
@@ -1460,7 +1461,7 @@ k_explicit_b(const TcDev* __restrict__ ds, const int2* __restrict__ emap, int k,
 // slot holds the mean flow U, W), 16 slots a block, a lane per component as in
 // k_solve.  (One thread per slot was the latency of six recurrences and an energy kernel
 // that read u, v, w again: a restart of 129x128x128 with its statistics, k_init with a
-// thread per pair included, 1662 -> 670 us.)
+// thread per pair included, 1662 -> 670 us, and 585 with the rows of k_init as they are.)
 //
 // First radial derivative of u, v and w, the operator of the energy budget: explicit
 // one-sided 5-point D on the walls (dwall) and on rows 1, Nr-2 (l1 rows with d0 = 1),
